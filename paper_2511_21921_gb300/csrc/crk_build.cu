@@ -612,7 +612,8 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
   }
   const R hi2 = sq(hi);
   // gather entries fill this lane's column from the front, scatter-only
-  // entries from the back; kg + ks > cap_pp means the column overflowed
+  // entries from the back (moved up at the end); kg + ks > cap_pp means the
+  // column overflowed
   int kg = 0, ks = 0;
   const int64_t wbase = w * cap_pp * 32 + lane;
   bool overflow = false;
@@ -918,9 +919,26 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
   if (overflow && lane == 0) set_status(hdr, CRK_ENOMEM);
   const int need = kg + ks;
   if (need > cap_pp) set_status(hdr, CRK_ENOMEM);
-  // counts that stay inside the column
-  const int cg = kg < cap_pp ? kg : (int)cap_pp;
-  const int cs = ks < cap_pp - cg ? ks : (int)(cap_pp - cg);
+  // a column that overflowed is left empty: its later slots were not written
+  const int cg = need <= cap_pp ? kg : 0;
+  const int cs = need <= cap_pp ? ks : 0;
+  // close the gap: move scatter-only entries from the back of the column to
+  // just behind the gather part, so that a union list is slots 0 .. cg + cs - 1
+  // (only the entries beyond the final end move, into slots no entry holds)
+  {
+    const int gap = (int)cap_pp - cg - cs;
+    const int mv = cs < gap ? cs : gap;
+    uint32_t* c0 = ell + wbase;
+    for (int t = 0; t < mv; t += 4) {
+      uint32_t e[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        e[q] = t + q < mv ? c0[(cap_pp - 1 - t - q) * 32] : 0u;
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        if (t + q < mv) c0[(int64_t)(cg + t + q) * 32] = e[q];
+    }
+  }
   if (live) {
     cnt_g[s] = cg;
     cnt_s[s] = cs;
@@ -968,8 +986,7 @@ __global__ void k_csr_fill(const int32_t* __restrict__ perm, const int32_t* __re
   const int ng = cg[s], ns = mode ? cs[s] : 0;
   const int64_t base = (s >> 5) * cap_pp * 32 + (s & 31);
   for (int k = 0; k < ng + ns; ++k) {
-    const int64_t slot = k < ng ? k : cap_pp - 1 - (k - ng);
-    const uint32_t e = ell[base + slot * 32];
+    const uint32_t e = ell[base + (int64_t)k * 32];
     const int32_t j = perm[e & kIdxMask];
     // insertion into the sorted prefix of this row
     int64_t pos = r0 + k;

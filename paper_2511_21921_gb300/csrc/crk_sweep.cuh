@@ -17,7 +17,7 @@ struct Common {
   const int32_t* __restrict__ boxid;
   const double* __restrict__ box_L;
   const int32_t* __restrict__ perm;
-  int64_t cap_pp;  // list slots per particle: gather part from the front, scatter-only from the back
+  int64_t cap_pp;  // list slots per particle: gather part, then the scatter-only entries
   int pf;          // prefetch distance in list entries (0 = off)
   // optional compacted work list of the active-set sweeps (sorted indices; its
   // length on the device): warps then take 32 listed particles per item
@@ -218,6 +218,10 @@ constexpr int sweep_regs(int block, int minb) {
 }
 
 
+// List entries are streamed from memory, so the plain-load mode reads them
+// this many steps before the record they name.
+constexpr int kAhead = 4;
+
 // Persistent sweep: warps pull 32-particle work items from an atomic queue --
 // 32 consecutive sorted particles, or 32 entries of a work list (the active
 // set's compacted list, or for passes with BALANCE the build's list ordered by
@@ -269,10 +273,7 @@ __global__ void __launch_bounds__(P::BLOCK) __maxnreg__(sweep_regs(P::BLOCK, MIN
       // union list (gather part, then scatter-only part) through the ring
       const int tot = lg + ls;
       const int wmax = __reduce_max_sync(kFull, tot);
-      auto entry = [&](int k) -> uint32_t {
-        const int64_t slot = k < lg ? k : a.c.cap_pp - 1 - (k - lg);
-        return __ldg(col + slot * 32);
-      };
+      auto entry = [&](int k) -> uint32_t { return __ldg(col + (int64_t)k * 32); };
       // a bad entry (bounds-checked build only) is redirected to the particle itself
       auto safe = [&](uint32_t e) -> uint32_t {
         return index_ok(a.c.hdr, e & kIdxMask, a.c.n) ? e : (uint32_t)s;
@@ -334,9 +335,7 @@ __global__ void __launch_bounds__(P::BLOCK) __maxnreg__(sweep_regs(P::BLOCK, MIN
       const int tot = lg + ls;
       const int wmax = P::GATHER && !its ? a.c.wlen_g[wi] : __reduce_max_sync(kFull, tot);
       auto raw = [&](int k) -> uint32_t {
-        if (k >= tot) return 0u;
-        const int64_t slot = k < lg ? k : a.c.cap_pp - 1 - (k - lg);
-        return __ldg(col + slot * 32);
+        return k < tot ? __ldg(col + (int64_t)k * 32) : 0u;
       };
       Real b0[D][P::SW0], b1[D][P::SW1 > 0 ? P::SW1 : 1];
       uint32_t eb[D], en[D];
@@ -368,9 +367,7 @@ __global__ void __launch_bounds__(P::BLOCK) __maxnreg__(sweep_regs(P::BLOCK, MIN
       const int tot = lg + ls;
       const int wmax = P::GATHER && !its ? a.c.wlen_g[wi] : __reduce_max_sync(kFull, tot);
       auto raw = [&](int k) -> uint32_t {
-        if (k >= tot) return 0u;
-        const int64_t slot = k < lg ? k : a.c.cap_pp - 1 - (k - lg);
-        return __ldg(col + slot * 32);
+        return k < tot ? __ldg(col + (int64_t)k * 32) : 0u;
       };
       uint32_t enext = raw(0);
       auto fetch = [&](int k, uint32_t& e, bool& ok, Real* r0, Real* r1) {
@@ -389,41 +386,26 @@ __global__ void __launch_bounds__(P::BLOCK) __maxnreg__(sweep_regs(P::BLOCK, MIN
         fetch(k + 2, ea, oka, A0, A1);
         if (okb) P::pair_s(a, st, B0, B1, eb & kIdxMask, eb);
       }
-    } else if (P::GATHER) {
-      // gather part only: the same row of every lane is one 128-byte line
-      const int wg = its ? __reduce_max_sync(kFull, lg) : a.c.wlen_g[wi];
-      const int pf = a.c.pf;
-      for (int k = 0; k < wg; ++k) {
-        if (pf && k + pf < lg)
-          prefetch_sources<P>(a, __ldg(col + (int64_t)(k + pf) * 32) & kIdxMask);
-        const uint32_t e = __ldg(col + (int64_t)k * 32);
-        if (k < lg && index_ok(a.c.hdr, e & kIdxMask, a.c.n)) {
-          Real r0[P::SW0], r1[P::SW1 > 0 ? P::SW1 : 1];
-          load_sources<P>(a, e & kIdxMask, r0, r1);
-          P::pair_s(a, st, r0, r1, e & kIdxMask, e);
-        }
-      }
     } else {
-      // gather part then scatter-only part as one list per lane, so the warp
-      // runs to its longest union list rather than to the sum of the longest
-      // parts
+      // plain loads: the record of entry k is loaded when its pair is
+      // evaluated
       const int tot = lg + ls;
-      const int wmax = __reduce_max_sync(kFull, tot);
-      const int pf = a.c.pf;
+      const int wmax = P::GATHER && !its ? a.c.wlen_g[wi] : __reduce_max_sync(kFull, tot);
+      uint32_t e[kAhead];
+      auto raw = [&](int k) -> uint32_t { return k < tot ? __ldg(col + (int64_t)k * 32) : 0u; };
+#pragma unroll
+      for (int i = 0; i < kAhead; ++i) e[i] = raw(i);
+      const bool pf = a.c.pf > 0;
       for (int k = 0; k < wmax; ++k) {
-        if (pf && k + pf < tot) {
-          const int kp = k + pf;
-          const int64_t sp = kp < lg ? kp : a.c.cap_pp - 1 - (kp - lg);
-          prefetch_sources<P>(a, __ldg(col + sp * 32) & kIdxMask);
-        }
-        if (k < tot) {
-          const int64_t slot = k < lg ? k : a.c.cap_pp - 1 - (k - lg);
-          const uint32_t e = __ldg(col + slot * 32);
-          if (index_ok(a.c.hdr, e & kIdxMask, a.c.n)) {
-            Real r0[P::SW0], r1[P::SW1 > 0 ? P::SW1 : 1];
-            load_sources<P>(a, e & kIdxMask, r0, r1);
-            P::pair_s(a, st, r0, r1, e & kIdxMask, e);
-          }
+        const uint32_t ek = e[0];
+#pragma unroll
+        for (int i = 0; i + 1 < kAhead; ++i) e[i] = e[i + 1];
+        e[kAhead - 1] = raw(k + kAhead);
+        if (pf && k + 1 < tot) prefetch_sources<P>(a, e[0] & kIdxMask);
+        if (k < tot && index_ok(a.c.hdr, ek & kIdxMask, a.c.n)) {
+          Real r0[P::SW0], r1[P::SW1 > 0 ? P::SW1 : 1];
+          load_sources<P>(a, ek & kIdxMask, r0, r1);
+          P::pair_s(a, st, r0, r1, ek & kIdxMask, ek);
         }
       }
     }
