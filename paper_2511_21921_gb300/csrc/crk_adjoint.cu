@@ -246,7 +246,6 @@ template <class R, bool VAR = false> struct PassA2 {
     const R* __restrict__ us;
     const R* __restrict__ Ds;
     const R* __restrict__ ms;
-    const R* __restrict__ coef;
     R* rec_a1;
     R* acc;
     R* cbar;
@@ -257,62 +256,122 @@ template <class R, bool VAR = false> struct PassA2 {
     R* dvdt;
     R* dudt;
   };
-  using D2 = P2<R>;
   struct State {
-    R ri[RC::C2];  // own record, columns negated (load_own_rates_record)
+    R ri[RC::C2];
     R ab[4];
-    R L, halfL;
+    R L, halfL, rho, cs;
     int64_t s;
-    // sums over the pairs; the factors that depend on this particle alone are
-    // applied in end()
-    D2 xb01, vb01;
-    R xb2, vb2;
-    R h1;        // -(1/h) times this is the h part through W, g and mu
-    R h2;        // -(1/h)^2 times this is the h part through eta
-    R Vb, Pb;    // Vb: times -1/2
-    R q1, q2;    // sum of Qb mu, of Qb mu^2
-    R u, ubs;    // specific energy and its cotangent through the energy split
-    D2 K[8];     // minus the cotangents of M's constant column; those of its others
-    D2 gvb00, gvb2;    // (00, 01), (02, 12)
-    R gvb11, gvb22;
+    R xb[3], vb[3], hb, Vb, Pb, rhob, cb;
+    R u, ubs;  // specific energy and its cotangent through the energy split
+    R Cb[16], gvb[9];
     R fa[3];
     Acc<R> fe;
   };
   __device__ static void begin(const Args& a, int64_t s, State& st) {
-    load_own_rates_record<R>(a.rec_c2, s, st.ri);
+    load_rec<RC::C2>(a.rec_c2, s, st.ri);
     load_rec<4>(a.rec_ab, s, st.ab);
     const double L = a.c.box_L[a.c.boxid[s]];
     st.L = (R)L;
     st.halfL = (R)(0.5 * L);
+    st.rho = a.rhos[s];
+    st.cs = sqrt_(a.ggm1 * a.us[s]);
     st.s = s;
-    const D2 zero = dup2(R(0));
-    st.xb01 = st.vb01 = st.gvb00 = st.gvb2 = zero;
-    st.xb2 = st.vb2 = st.h1 = st.h2 = st.Vb = st.Pb = st.q1 = st.q2 = R(0);
-    st.gvb11 = st.gvb22 = R(0);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) st.xb[k] = st.vb[k] = R(0);
+    st.hb = st.Vb = st.Pb = st.rhob = st.cb = R(0);
     st.u = VAR ? a.us[s] : R(0);
     st.ubs = R(0);
 #pragma unroll
-    for (int k = 0; k < 8; ++k) st.K[k] = zero;
+    for (int k = 0; k < 16; ++k) st.Cb[k] = R(0);
+#pragma unroll
+    for (int k = 0; k < 9; ++k) st.gvb[k] = R(0);
     st.fa[0] = st.fa[1] = st.fa[2] = R(0);
     st.fe = Acc<R>();
   }
   __device__ static const R* src0(const Args& a) { return a.rec_c2; }
   __device__ static const R* src1(const Args& a) { return a.rec_ab; }
-  // (grad v + grad v^T) e from grad v e
-  __device__ static __forceinline__ void both_gradv(const R* rec, const R* e, const R* gve, R* o) {
-#pragma unroll
-    for (int q = 0; q < 3; ++q)
-      o[q] = fma_(rec[c2_gv(2, q)], e[2],
-                  fma_(rec[c2_gv(1, q)], e[1], fma_(rec[c2_gv(0, q)], e[0], gve[q])));
-  }
   __device__ static void pair_s(const Args& a, State& st, const R* rj, const R* abj, uint32_t j,
                                 uint32_t) {
     const R* ri = st.ri;
-    PairC2<R> p;
-    p.template forward<VAR>(ri, rj, st.L, st.halfL, a.av);
+    R d[3];
+    separation(ri, rj, st.L, st.halfL, d);
+    const R r2 = dot3(d, d);
+    const R r = radius(r2);
+    const bool rk = ri[RC::C2_FLAG] == R(0) && rj[RC::C2_FLAG] == R(0);
+    const R ihi = ri[RC::C2_IH], ihj = rj[RC::C2_IH];
+    // ---- forward recompute (the expressions of PairC2::force)
+    R Wi, gi, Wj, gj;
+    wendland(r, ihi, Wi, gi);
+    wendland(r, ihj, Wj, gj);
+    const R nd[3] = {-d[0], -d[1], -d[2]};
+    R Gi[3], Gj[3];
+    rk_gradient(ri + RC::C2_A, d, Wi, gi, rk, Gi);
+    rk_gradient(rj + RC::C2_A, nd, Wj, gj, rk, Gj);
+    const R* gvi = ri + RC::C2_GV;
+    const R* gvj = rj + RC::C2_GV;
+    R gix[3], gjx[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      gix[p] = gvi[3 * p] * d[0] + gvi[3 * p + 1] * d[1] + gvi[3 * p + 2] * d[2];
+      gjx[p] = gvj[3 * p] * d[0] + gvj[3 * p + 1] * d[1] + gvj[3 * p + 2] * d[2];
+    }
+    R phi = R(0), phi0 = R(0), damp = R(1), z = R(0), pa = R(0), pb = R(0);
+    bool dampon = false;
+    const R ihmin = fmin(ihi, ihj);
+    const R eta = r * ihmin;
+    if (a.av.limiter) {
+      pa = d[0] * gix[0] + d[1] * gix[1] + d[2] * gix[2];
+      pb = d[0] * gjx[0] + d[1] * gjx[1] + d[2] * gjx[2];
+      phi0 = PairC2<R>::limiter_phi(pa, pb);
+      phi = phi0;
+      if (eta < a.av.eta_crit) {
+        dampon = true;
+        z = (eta - a.av.eta_crit) / a.av.eta_fold;
+        damp = exp_(-(z * z));
+        phi = phi0 * damp;
+      }
+    }
+    const R hphi = R(0.5) * phi;
+    R vij[3], vh[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      vij[p] = ri[RC::C2_VEL + p] - rj[RC::C2_VEL + p];
+      vh[p] = vij[p] - hphi * (gix[p] + gjx[p]);
+    }
+    const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
+    const R Di = r2 * (ihi * ihi) + a.av.eps2;
+    const R Dj = r2 * (ihj * ihj) + a.av.eps2;
+    const R tmi = vx * ihi / Di, tmj = vx * ihj / Dj;
+    const R mui = tmi < R(0) ? tmi : R(0);
+    const R muj = tmj < R(0) ? tmj : R(0);
+    const R qai = ri[RC::C2_QA], qbi = ri[RC::C2_QB], qaj = rj[RC::C2_QA], qbj = rj[RC::C2_QB];
+    const R Qi = mui * (qbi * mui - qai);
+    const R Qj = muj * (qbj * muj - qaj);
+    const R ViVj = ri[RC::C2_V] * rj[RC::C2_V];
     const bool qside = VAR && a.av.q_side;
-    R f = R(0.5), dfdui = R(0), E = R(0);
-    if (VAR || a.dvdt) E = p.work();
+    R Pi = R(0), pre = R(0), VV = R(0), PP = R(0);
+    R F[3], dG[3];
+    if (qside) {  // the expressions of PairC2::force, per-side viscosity
+      VV = R(-0.5) * ViVj;
+      PP = ri[RC::C2_P] + rj[RC::C2_P];
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        dG[p] = Gi[p] - Gj[p];
+        const R qg = rsub(rmul(Qi, Gi[p]), rmul(Qj, Gj[p]));
+        F[p] = VV * radd(rmul(PP, dG[p]), R(2) * qg);
+      }
+    } else {
+      Pi = (ri[RC::C2_P] + rj[RC::C2_P]) + (Qi + Qj);
+      pre = R(-0.5) * ViVj * Pi;
+#pragma unroll
+      for (int p = 0; p < 3; ++p) {
+        dG[p] = Gi[p] - Gj[p];
+        F[p] = pre * dG[p];
+      }
+    }
+    // pair work E_ij = F.(v_j - v_i) and i's share f_ij of it
+    const R E = -(F[0] * vij[0] + F[1] * vij[1] + F[2] * vij[2]);
+    R f = R(0.5), dfdui = R(0);
     if (VAR && a.av.energy_split) {
       const R uj = a.us[j];
       f = energy_share(true, E, st.u, uj);
@@ -321,156 +380,125 @@ template <class R, bool VAR = false> struct PassA2 {
     }
     if (a.dvdt) {  // forward rates from the same force (fused sweep)
 #pragma unroll
-      for (int k = 0; k < 3; ++k) st.fa[k] += p.F[k];
+      for (int p = 0; p < 3; ++p) st.fa[p] += F[p];
       st.fe.add(f * E);
     }
-    // beta = g_dudt / (2 m), so the energy term of the pair is c E with
-    // c = 2 (beta_i f_ij + beta_j f_ji) (beta_i + beta_j for halves)
-    R csum;
-    if (VAR && a.av.energy_split) {
-      csum = R(2) * (st.ab[3] * f + abj[3] * (R(1) - f));
-      st.ubs += R(2) * (st.ab[3] - abj[3]) * E * dfdui;
-    } else {
-      csum = st.ab[3] + abj[3];
-    }
-    R Fb[3];
+    // ---- reverse.  beta = g_dudt / (2 m), so the energy term of the pair is
+    // c E with c = 2 (beta_i f_ij + beta_j f_ji) (beta_i + beta_j for halves)
+    const R csum = R(2) * (st.ab[3] * f + abj[3] * (R(1) - f));
+    if (VAR && a.av.energy_split) st.ubs += R(2) * (st.ab[3] - abj[3]) * E * dfdui;
+    R Fb[3], vijb[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) Fb[k] = fma_(-csum, p.vij[k], st.ab[k] - abj[k]);
-    // cotangents of G_i (qi) and, negated, of G_j (qj), and of Q_i, Q_j
-    R qi[3], qj[3], Qib, Qjb;
-    const R Vj = rj[RC::C2_V];
+    for (int p = 0; p < 3; ++p) {
+      Fb[p] = (st.ab[p] - abj[p]) - csum * vij[p];
+      vijb[p] = -csum * F[p];
+    }
+    R Gib[3], Gjb[3], Qib, Qjb;
     if (qside) {
       // F = VV [PP dG + 2 (Q_i G_i - Q_j G_j)]
       R VVb = R(0), FdG = R(0), FGi = R(0), FGj = R(0);
 #pragma unroll
-      for (int k = 0; k < 3; ++k) {
-        VVb += Fb[k] * (p.PP * p.dG[k] + R(2) * (p.Qi * p.Gi[k] - p.Qj * p.Gj[k]));
-        FdG += Fb[k] * p.dG[k];
-        FGi += Fb[k] * p.Gi[k];
-        FGj += Fb[k] * p.Gj[k];
-        qi[k] = p.VV * (p.PP + R(2) * p.Qi) * Fb[k];
-        qj[k] = p.VV * (p.PP + R(2) * p.Qj) * Fb[k];
+      for (int p = 0; p < 3; ++p) {
+        VVb += Fb[p] * (PP * dG[p] + R(2) * (Qi * Gi[p] - Qj * Gj[p]));
+        FdG += Fb[p] * dG[p];
+        FGi += Fb[p] * Gi[p];
+        FGj += Fb[p] * Gj[p];
+        Gib[p] = VV * (PP + R(2) * Qi) * Fb[p];
+        Gjb[p] = -VV * (PP + R(2) * Qj) * Fb[p];
       }
-      Qib = R(2) * p.VV * FGi;
-      Qjb = R(-2) * p.VV * FGj;
-      st.Vb = fma_(VVb, Vj, st.Vb);
-      st.Pb += p.VV * FdG;
+      Qib = R(2) * VV * FGi;
+      Qjb = R(-2) * VV * FGj;
+      st.Vb += VVb * (R(-0.5) * rj[RC::C2_V]);
+      st.Pb += VV * FdG;
     } else {
-      const R preb = dot3(Fb, p.dG);
-      const R pre = p.VV * p.Pi;
-      const R pv = preb * Vj;
+      const R preb = Fb[0] * dG[0] + Fb[1] * dG[1] + Fb[2] * dG[2];
 #pragma unroll
-      for (int k = 0; k < 3; ++k) qi[k] = pre * Fb[k];
-      qj[0] = qi[0];
-      qj[1] = qi[1];
-      qj[2] = qi[2];
-      st.Vb = fma_(pv, p.Pi, st.Vb);
-      Qib = Qjb = pv * (R(-0.5) * ri[RC::C2_V]);
-      st.Pb += Qib;
+      for (int p = 0; p < 3; ++p) {
+        Gib[p] = pre * Fb[p];
+        Gjb[p] = -Gib[p];
+      }
+      const R Pib = preb * (R(-0.5) * ViVj);
+      st.Vb += preb * (R(-0.5) * rj[RC::C2_V] * Pi);
+      st.Pb += Pib;
+      Qib = Qjb = Pib;
     }
-    // ---- viscosity: Q = mu (QB mu + QA'), mu = min(0, t), t = vx ih / D
-    R mui, muj, ti, tj;
-    get2(p.mu, mui, muj);
-    get2(p.t, ti, tj);
-    const R y1 = Qib * mui;
-    st.q1 += y1;
-    st.q2 = fma_(y1, mui, st.q2);
-    R mbi, mbj;
-    get2(mul2(mk2(Qib, Qjb), fma2(mk2(ri[RC::C2_QB], rj[RC::C2_QB]), p.mu, p.qs)), mbi, mbj);
-    const D2 mb = mk2(ti < R(0) ? mbi : R(0), tj < R(0) ? mbj : R(0));
-    const R vxb = hadd2(mul2(mb, p.hD));
-    // dt/d(r^2) = -t ih^2/D, dt/d(ih) = (t/ih) (1 - 2 r^2 ih^2/D)
-    const D2 zt = mul2(mb, p.t);
-    const D2 zw = mul2(zt, mul2(p.ih2, p.iD));
-    const R r2b = -hadd2(zw);
-    const R h1a = fma_(R(-2) * p.r2, lo2(zw), lo2(zt));
-    // ---- limiter: vx = v_ij.d - phi (pa + pb)/2
-    const R sm = p.pa + p.pb;
-    const R hphi = R(-0.5) * p.phi;
-    const R phib = R(-0.5) * (vxb * sm);
-    R ki = vxb * hphi, kj = ki, rb = R(0);  // cotangents of pa and pb
+    const R muib = Qib * (R(2) * qbi * mui - qai);
+    const R mujb = Qjb * (R(2) * qbj * muj - qaj);
+    st.rhob += Qib * mui * (a.Cq * mui - a.Cl * st.cs);
+    st.cb += Qib * mui * (-a.Cl * st.rho);
+    R vxb = R(0), r2b = R(0), ihib = R(0), rb = R(0);
+    R db[3] = {R(0), R(0), R(0)};
+    if (tmi < R(0)) {
+      vxb += muib * ihi / Di;
+      ihib += muib * (vx / Di) * (R(1) - R(2) * r2 * (ihi * ihi) / Di);
+      r2b += muib * (-vx * (ihi * ihi * ihi) / (Di * Di));
+    }
+    if (tmj < R(0)) {
+      vxb += mujb * ihj / Dj;
+      r2b += mujb * (-vx * (ihj * ihj * ihj) / (Dj * Dj));
+    }
+    R vhb[3], gsum[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      vhb[p] = vxb * d[p];
+      db[p] += vxb * vh[p];
+      vijb[p] += vhb[p];
+      gsum[p] = gix[p] + gjx[p];
+    }
+    const R phib = R(-0.5) * (vhb[0] * gsum[0] + vhb[1] * gsum[1] + vhb[2] * gsum[2]);
+    R gixb[3], gjxb[3];
+#pragma unroll
+    for (int p = 0; p < 3; ++p) gixb[p] = gjxb[p] = -hphi * vhb[p];
     if (a.av.limiter) {
-      // d phi0/d pa = 4 pb (pb - pa)/(pa + pb)^3
-      const R c4 = R(4) * (phib * p.damp) * p.is * ((p.pb - p.pa) * p.is);
-      ki = fma_(c4, p.pb * p.is, ki);
-      kj = fma_(-c4, p.pa * p.is, kj);
-      // eta = r min(1/h_i, 1/h_j), z = (eta - eta_crit)/eta_fold where negative
-      const R etab = phib * p.phi * (R(-2) * p.z) * a.av.inv_fold;
-      rb = etab * p.ihmin;
-      const R ihi = ri[RC::C2_IH], ihj = rj[RC::C2_IH];
-      const bool own = (ihi < ihj) || (ihi == ihj && st.s < (int64_t)j);
-      st.h2 = fma_(own ? etab : R(0), p.r, st.h2);
-    }
-    // grad v cotangent k_i d d^T, symmetric
-    const D2 ke01 = mul2(dup2(ki), p.e01);
-    const R ke2 = ki * p.e[2];
-    st.gvb00 = fma2(dup2(lo2(ke01)), p.e01, st.gvb00);
-    st.gvb2 = fma2(ke01, p.e2, st.gvb2);
-    st.gvb11 = fma_(hi2(ke01), p.e[1], st.gvb11);
-    st.gvb22 = fma_(ke2, p.e[2], st.gvb22);
-    R wi[3], wj[3];
-    both_gradv(ri, p.e, p.gie, wi);
-    both_gradv(rj, p.e, p.gje, wj);
-    // ---- corrected gradients: Y = minus the cotangent of (u, lin) of i, plus j's
-    R Wi, Wj, gi, gj;
-    get2(p.W, Wi, Wj);
-    get2(p.g, gi, gj);
-    const R tei = dot3(qi, p.e), tej = qside ? dot3(qj, p.e) : tei;
-    const D2 qi01 = mk2(qi[0], qi[1]), qj01 = mk2(qj[0], qj[1]);
-    D2 Yi01 = mul2(dup2(-Wi), qi01), Yi2l = mk2(-Wi * qi[2], gi * tei);
-    D2 Yj01 = mul2(dup2(Wj), qj01), Yj2l = mk2(Wj * qj[2], gj * tej);
-    if (a.av.relax && !(ri[RC::C2_FLAG] == R(0) && rj[RC::C2_FLAG] == R(0)))
-      Yi01 = Yi2l = Yj01 = Yj2l = dup2(R(0));
-    // cotangents of W: q.u for i, -q.u for j; of g: -lin (q.e) for both
-    const R Wib = fma_(lo2(p.ui2l), qi[2], hadd2(mul2(p.ui01, qi01)));
-    const R Wjb = -fma_(lo2(p.uj2l), qj[2], hadd2(mul2(p.uj01, qj01)));
-    const D2 Wb = mk2(Wib, Wjb);
-    const D2 gb = mk2(-hi2(p.ui2l) * tei, -hi2(p.uj2l) * tej);
-    // gg = (1/r) dg/dr = -30 c_g / h^7 (1-q)^4
-    const D2 gg = mul2(mul2(mul2(p.ih2, mul2(p.ih2, p.ih2)), mul2(p.ih, p.om4)),
-                       dup2(R(-30.0 * Wend<R>::cg)));
-    const D2 cr = fma2(gb, gg, mul2(Wb, p.g));
-    st.h1 += h1a + fma_(Wib, fma_(gi, p.r2, R(3) * Wi),
-                        lo2(gb) * fma_(lo2(gg), p.r2, R(5) * gi));
-    // everything along e (d = -e): W, g, the viscosity's r^2 and eta's r
-    const R along = -(hadd2(cr) + fma_(R(2), r2b, rb * p.ir));
-    const D2 ea[3] = {p.e0, p.e1, p.e2};
-    st.K[0] = add2(st.K[0], Yi01);
-    st.K[1] = add2(st.K[1], Yi2l);
-    R Yx[3];
+      R phi0b = phib;
+      if (dampon) {
+        phi0b = phib * damp;
+        const R dampb = phib * phi0;
+        const R zb = dampb * (R(-2) * z * damp);
+        const R etab = zb / a.av.eta_fold;
+        rb += etab * ihmin;
+        const bool own = (ihi < ihj) || (ihi == ihj && st.s < (int64_t)j);
+        if (own) ihib += etab * r;
+      }
+      if (pa * pb > R(0)) {
+        const R sm = pa + pb;
+        const R s3 = sm * sm * sm;
+        const R pab = phi0b * R(4) * pb * (pb - pa) / s3;
+        const R pbb = phi0b * R(4) * pa * (pa - pb) / s3;
 #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      const R* Mi = ri + RC::C2_M + 4 + 4 * k;
-      const R* Mj = rj + RC::C2_M + 4 + 4 * k;
-      Yx[k] = hadd2(fma2(mk2(Mj[2], Mj[3]), Yj2l,
-                         fma2(mk2(Mj[0], Mj[1]), Yj01,
-                              fma2(mk2(Mi[2], Mi[3]), Yi2l, mul2(mk2(Mi[0], Mi[1]), Yi01)))));
-      st.K[2 + 2 * k] = fma2(Yi01, ea[k], st.K[2 + 2 * k]);
-      st.K[3 + 2 * k] = fma2(Yi2l, ea[k], st.K[3 + 2 * k]);
+        for (int p = 0; p < 3; ++p) {
+          db[p] += pab * gix[p] + pbb * gjx[p];
+          gixb[p] += pab * d[p];
+          gjxb[p] += pbb * d[p];
+        }
+      }
     }
-    R gq[3];
-    if (qside) {
 #pragma unroll
-      for (int k = 0; k < 3; ++k) gq[k] = p.gli * qi[k] + p.glj * qj[k];
-    } else {
-      const R gl = p.gli + p.glj;
+    for (int p = 0; p < 3; ++p)
 #pragma unroll
-      for (int k = 0; k < 3; ++k) gq[k] = gl * qi[k];
+      for (int q = 0; q < 3; ++q) {
+        st.gvb[3 * p + q] += gixb[p] * d[q];
+        db[q] += gvi[3 * p + q] * gixb[p] + gvj[3 * p + q] * gjxb[p];
+      }
+    R Wib = R(0), gib = R(0), Wjb = R(0), gjb = R(0);
+    R ndb[3] = {R(0), R(0), R(0)};
+    R Cjb[16];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) Cjb[k] = R(0);
+    rk_gradient_rev(ri + RC::C2_A, d, Wi, gi, rk, Gib, st.Cb, db, Wib, gib);
+    rk_gradient_rev(rj + RC::C2_A, nd, Wj, gj, rk, Gjb, Cjb, ndb, Wjb, gjb);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) db[p] -= ndb[p];
+    st.hb += wendland_rev(Wib, gib, Wi, gi, wendland_gg(r, ihi), r2, ihi, d, db);
+    (void)wendland_rev(Wjb, gjb, Wj, gj, wendland_gg(r, ihj), r2, ihj, d, db);
+    const R rr = (r > R(0)) ? rb / r : R(0);
+#pragma unroll
+    for (int p = 0; p < 3; ++p) {
+      db[p] += (rr + R(2) * r2b) * d[p];
+      st.xb[p] += db[p];
+      st.vb[p] += vijb[p];
     }
-    const D2 w01i = mk2(wi[0], wi[1]), w01j = mk2(wj[0], wj[1]);
-    const D2 vij01 = mk2(p.vij[0], p.vij[1]);
-    D2 db01 = add2(mk2(Yx[0], Yx[1]), mk2(gq[0], gq[1]));
-    db01 = fma2(dup2(vxb), vij01, db01);
-    db01 = fma2(dup2(-ki), w01i, db01);
-    db01 = fma2(dup2(-kj), w01j, db01);
-    db01 = fma2(dup2(along), p.e01, db01);
-    st.xb01 = add2(st.xb01, db01);
-    const R db2 = fma_(along, p.e[2],
-                       fma_(-kj, wj[2], fma_(-ki, wi[2], fma_(vxb, p.vij[2], Yx[2] + gq[2]))));
-    st.xb2 += db2;
-    // v_ij enters through vx (along d) and the pair work
-    st.vb01 = fma2(dup2(-vxb), p.e01, fma2(dup2(-csum), mk2(p.F[0], p.F[1]), st.vb01));
-    st.vb2 = fma_(-vxb, p.e[2], fma_(-csum, p.F[2], st.vb2));
+    st.hb += ihib * (-(ihi * ihi));
   }
   __device__ static void end(const Args& a, int64_t s, State& st) {
     using A_ = ARec<R>;
@@ -481,84 +509,44 @@ template <class R, bool VAR = false> struct PassA2 {
       for (int k = 0; k < 3; ++k) a.dvdt[k * a.c.n + p] = st.fa[k] * im;
       a.dudt[p] = st.fe.s * im;
     }
-    const R u = a.us[s], rho = a.rhos[s];
-    const R cs = sqrt_(a.ggm1 * u);
-    // Q = rho (Cq mu^2 - Cl c mu); EOS: P = (gamma-1) rho u, c = sqrt(gamma (gamma-1) u)
-    const R rhob = a.Cq * st.q2 - a.Cl * cs * st.q1 + a.gm1 * u * st.Pb;
-    const R cb = -a.Cl * rho * st.q1;
-    const R ub = a.gm1 * rho * st.Pb + (cs > R(0) ? cb * a.ggm1 / (R(2) * cs) : R(0)) + st.ubs;
+    const R u = a.us[s];
+    // EOS: P = (gamma-1) rho u, c = sqrt(gamma (gamma-1) u)
+    const R rhob = st.rhob + a.gm1 * u * st.Pb;
+    const R ub = a.gm1 * st.rho * st.Pb + (st.cs > R(0) ? st.cb * a.ggm1 / (R(2) * st.cs) : R(0)) +
+                 st.ubs;
     // rho = N / D
     const R D = a.Ds[s];
-    const R Nb = rhob / D, Db = -rhob * rho / D;
-    R C[16];
-    load_rec<16>(a.coef, s, C);
-    const R ih = st.ri[RC::C2_IH];
+    const R Nb = rhob / D, Db = -rhob * st.rho / D;
     R r[A_::A1];
 #pragma unroll
     for (int k = 0; k < A_::A1; ++k) r[k] = R(0);
 #pragma unroll
-    for (int k = 0; k < RC::XW; ++k) r[k] = st.ri[RC::C2_X + k];
-    r[A_::A1_IH] = ih;
+    for (int k = 0; k < RC::XW; ++k) r[k] = st.ri[k];
+    r[A_::A1_IH] = st.ri[RC::C2_IH];
     r[A_::A1_V] = st.ri[RC::C2_V];
     r[A_::A1_M] = a.ms[s];
 #pragma unroll
     for (int k = 0; k < 3; ++k) r[A_::A1_VEL + k] = st.ri[RC::C2_VEL + k];
 #pragma unroll
-    for (int k = 0; k < 16; ++k) r[A_::A1_C + k] = C[k];
+    for (int k = 0; k < 16; ++k) r[A_::A1_C + k] = st.ri[RC::C2_A + k];
     r[A_::A1_NB] = Nb;
     r[A_::A1_DB] = Db;
-    R gvb[9];
-    get2(st.gvb00, gvb[0], gvb[1]);
-    get2(st.gvb2, gvb[2], gvb[5]);
-    gvb[3] = gvb[1];
-    gvb[6] = gvb[2];
-    gvb[7] = gvb[5];
-    gvb[4] = st.gvb11;
-    gvb[8] = st.gvb22;
 #pragma unroll
-    for (int k = 0; k < 9; ++k) r[A_::A1_GVB + k] = gvb[k];
+    for (int k = 0; k < 9; ++k) r[A_::A1_GVB + k] = st.gvb[k];
     store_rec<A_::A1>(a.rec_a1, s, r);
     R ac[A_::ACC];
 #pragma unroll
     for (int k = 0; k < A_::ACC; ++k) ac[k] = R(0);
-    get2(st.xb01, ac[A_::XB], ac[A_::XB + 1]);
-    ac[A_::XB + 2] = st.xb2;
-    get2(st.vb01, ac[A_::VB], ac[A_::VB + 1]);
-    ac[A_::VB + 2] = st.vb2;
-    ac[A_::HB] = -ih * (st.h1 + ih * st.h2);
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      ac[A_::XB + k] = st.xb[k];
+      ac[A_::VB + k] = st.vb[k];
+    }
+    ac[A_::HB] = st.hb;
     ac[A_::UB] = ub;
-    ac[A_::VVB] = R(-0.5) * st.Vb;
+    ac[A_::VVB] = st.Vb;
     store_rec<A_::ACC>(a.acc, s, ac);
-    // cotangents of c_k = dA_k + A B_k, E_ka = A dB_ka + dA_k B_a, b_a = A B_a and
-    // lin's constant A, taken to those of A, B, grad A, grad B (C[7 + 3 k + a])
-    R cc[4], cm[3][4], Cb[16];
-    get2(st.K[0], cc[0], cc[1]);
-    get2(st.K[1], cc[2], cc[3]);
-#pragma unroll
-    for (int k = 0; k < 4; ++k) cc[k] = -cc[k];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      get2(st.K[2 + 2 * k], cm[k][0], cm[k][1]);
-      get2(st.K[3 + 2 * k], cm[k][2], cm[k][3]);
-    }
-    R Ab = cc[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-      R t = cc[k];
-      Ab += cc[k] * C[1 + k] + cm[k][3] * C[1 + k];
-      R bb = C[0] * (cc[k] + cm[k][3]);
-#pragma unroll
-      for (int q = 0; q < 3; ++q) {
-        t += cm[q][k] * C[1 + q];         // E_kq's share of dA_k
-        bb += cm[k][q] * C[4 + q];        // E_qk's share of B_k
-        Ab += cm[q][k] * C[7 + 3 * k + q];
-        Cb[7 + 3 * k + q] = C[0] * cm[q][k];
-      }
-      Cb[4 + k] = t;
-      Cb[1 + k] = bb;
-    }
-    Cb[0] = Ab;
-    store_rec<16>(a.cbar, s, Cb);
+    store_rec<16>(a.cbar, s, st.Cb);
   }
 };
 
@@ -991,7 +979,6 @@ crk_status adjoint_impl(Plan* plan, cudaStream_t st, char* ws, const R* v, const
                               reinterpret_cast<const R*>(ws + Ly.us),
                               reinterpret_cast<const R*>(ws + Ly.Ds),
                               ms,
-                              reinterpret_cast<const R*>(ws + Ly.coef),
                               rec_a1,
                               acc,
                               cbar,

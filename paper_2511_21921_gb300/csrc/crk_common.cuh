@@ -106,20 +106,12 @@ template <class R> struct Rec {
   // C1_VGW: the volume over gas and wind, negative for a wind particle
   static constexpr int C1_V = XW, C1_M = XW + 1, C1_VEL = XW + 2, C1_VGW = XW + 5,
                        C1 = round_up(XW + 6, VEC / 2);
-  // c2 (rates): the corrected kernel's gradient in the form the pair sweeps use
-  // it, M = four columns of four words,
-  //   const: c_k = dA_k + A B_k (k < 3), A;  column a: E_ka = A d_k B_a + dA_k B_a, A B_a,
-  // so that (u, lin) = const + sum_a column_a x_a gives grad W^R = W u + g lin x
-  // with lin = A (1 + B.x); then grad v (pairs of rows 0 and 1 per column, then
-  // row 2), 1/h, v, V, P, -C_l rho c, C_q rho, flag and x.  Words that are
-  // used together sit in even-odd pairs for the packed arithmetic (P2).
-  static constexpr int C2_M = 0, C2_GV = 16, C2_IH = 25, C2_VEL = 26, C2_V = 29, C2_P = 30,
-                       C2_QA = 31, C2_QB = 32, C2_FLAG = 33, C2_X = 34,
-                       C2 = round_up(34 + XW, VEC);
+  // c2 (rates): x, ih, V, P, qa, qb, flag, v[3], A, B[3], dA[3], dB[9], gv[9]
+  static constexpr int C2_IH = XW, C2_V = XW + 1, C2_P = XW + 2, C2_QA = XW + 3,
+                       C2_QB = XW + 4, C2_FLAG = XW + 5, C2_VEL = XW + 6, C2_A = XW + 9,
+                       C2_B = XW + 10, C2_DA = XW + 13, C2_DB = XW + 16, C2_GV = XW + 25,
+                       C2 = round_up(XW + 34, VEC);
 };
-
-// Column-pair order of the velocity gradient in a c2 record: word of gv[p][q].
-__host__ __device__ constexpr int c2_gv(int p, int q) { return p < 2 ? 16 + 2 * q + p : 22 + q; }
 
 // Records of the reverse sweeps (adjoint), same conventions as Rec.
 template <class R> struct ARec {
@@ -237,95 +229,13 @@ __device__ __forceinline__ double radd(double a, double b) { return __dadd_rn(a,
 __device__ __forceinline__ float rsub(float a, float b) { return __fsub_rn(a, b); }
 __device__ __forceinline__ double rsub(double a, double b) { return __dsub_rn(a, b); }
 
-// 1/sqrt(x) and 1/x: one MUFU instruction in float (about 1 ulp), full
-// precision in double
-__device__ __forceinline__ float rsqrt_(float x) {
-  float y;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
-__device__ __forceinline__ float rcp_(float x) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
-  return y;
-}
-__device__ __forceinline__ double rcp_(double x) { return 1.0 / x; }
-__device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
-// exp(-z^2)
-__device__ __forceinline__ float gauss_(float z) { return exp2f(z * (z * -1.4426950408889634f)); }
-__device__ __forceinline__ double gauss_(double z) { return exp(-(z * z)); }
+template <class R> __device__ __forceinline__ R rsqrt_(R x);
+template <> __device__ __forceinline__ float rsqrt_(float x) { return rsqrtf(x); }
+template <> __device__ __forceinline__ double rsqrt_(double x) { return rsqrt(x); }
 __device__ __forceinline__ float sqrt_(float x) { return sqrtf(x); }
 __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
 __device__ __forceinline__ float exp_(float x) { return expf(x); }
 __device__ __forceinline__ double exp_(double x) { return exp(x); }
-
-// ---------------------------------------------------------------------------
-// Pairs of reals.  In float one instruction (fma.rn.f32x2 and its relatives)
-// works on both: it takes one issue slot instead of two for the same FP32 pipe
-// time (measured on GB300: 75 TFLOP/s of packed against 79 of scalar fused
-// multiply-adds), and the pair sweeps are bound by issue, not by the pipe.
-// Every half rounds as the scalar operation does.  In double the two halves are
-// plain operations.
-// ---------------------------------------------------------------------------
-template <class R> struct P2;
-template <> struct P2<float> {
-  unsigned long long v;
-};
-template <> struct P2<double> {
-  double a, b;
-};
-__device__ __forceinline__ P2<float> mk2(float lo, float hi) {
-  P2<float> r;
-  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
-  return r;
-}
-__device__ __forceinline__ P2<double> mk2(double lo, double hi) { return P2<double>{lo, hi}; }
-__device__ __forceinline__ void get2(P2<float> p, float& lo, float& hi) {
-  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p.v));
-}
-__device__ __forceinline__ void get2(P2<double> p, double& lo, double& hi) { lo = p.a; hi = p.b; }
-template <class R> __device__ __forceinline__ R lo2(P2<R> p) {
-  R a, b;
-  get2(p, a, b);
-  return a;
-}
-template <class R> __device__ __forceinline__ R hi2(P2<R> p) {
-  R a, b;
-  get2(p, a, b);
-  return b;
-}
-template <class R> __device__ __forceinline__ R hadd2(P2<R> p) {
-  R a, b;
-  get2(p, a, b);
-  return a + b;
-}
-template <class R> __device__ __forceinline__ P2<R> dup2(R x) { return mk2(x, x); }
-__device__ __forceinline__ P2<float> add2(P2<float> a, P2<float> b) {
-  P2<float> r;
-  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
-__device__ __forceinline__ P2<float> mul2(P2<float> a, P2<float> b) {
-  P2<float> r;
-  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
-  return r;
-}
-__device__ __forceinline__ P2<float> fma2(P2<float> a, P2<float> b, P2<float> c) {
-  P2<float> r;
-  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
-  return r;
-}
-__device__ __forceinline__ P2<double> add2(P2<double> a, P2<double> b) {
-  return P2<double>{a.a + b.a, a.b + b.b};
-}
-__device__ __forceinline__ P2<double> mul2(P2<double> a, P2<double> b) {
-  return P2<double>{a.a * b.a, a.b * b.b};
-}
-__device__ __forceinline__ P2<double> fma2(P2<double> a, P2<double> b, P2<double> c) {
-  return P2<double>{__fma_rn(a.a, b.a, c.a), __fma_rn(a.b, b.b, c.b)};
-}
 
 // r = |x| from r^2 (0 for coincident points)
 template <class R> __device__ __forceinline__ R radius(R r2) {

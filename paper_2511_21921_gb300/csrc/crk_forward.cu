@@ -325,9 +325,23 @@ template <class R> struct PassC1 {
     const R div = st.gv[0] + st.gv[4] + st.gv[8];
     const bool flag = a.relax_dt > R(0) && exp_(fabs(div) * a.relax_dt) > R(8);
     R r[RC::C2];
-    // flag 0: corrected, 1: relaxed (App. A.1), 2: wind (no hydro force)
-    make_rates_record<R>(r, st.x, st.C, st.gv, st.ih, st.v, st.V, P, a.Cl * rho * cs, a.Cq * rho,
-                         st.wind ? R(2) : (flag ? R(1) : R(0)));
+#pragma unroll
+    for (int k = 0; k < RC::C2; ++k) r[k] = R(0);
+#pragma unroll
+    for (int k = 0; k < RC::XW; ++k) r[k] = st.x[k];
+    r[RC::C2_IH] = st.ih;
+    r[RC::C2_V] = st.V;
+    r[RC::C2_P] = P;
+    r[RC::C2_QA] = a.Cl * rho * cs;
+    r[RC::C2_QB] = a.Cq * rho;
+    // 0: corrected, 1: relaxed (App. A.1), 2: wind (no hydro force)
+    r[RC::C2_FLAG] = st.wind ? R(2) : (flag ? R(1) : R(0));
+#pragma unroll
+    for (int k = 0; k < 3; ++k) r[RC::C2_VEL + k] = st.v[k];
+#pragma unroll
+    for (int k = 0; k < 16; ++k) r[RC::C2_A + k] = st.C[k];
+#pragma unroll
+    for (int k = 0; k < 9; ++k) r[RC::C2_GV + k] = st.gv[k];
     store_rec<RC::C2>(a.rec_c2, s, r);
     a.rhos[s] = rho;
     a.Ds[s] = st.den.s;
@@ -378,7 +392,7 @@ template <class R, bool VAR = false> struct PassC2 {
     Acc<R> e;
   };
   __device__ static void begin(const Args& a, int64_t s, State& st) {
-    load_own_rates_record<R>(a.rec_c2, s, st.ri);
+    load_rec<RC::C2>(a.rec_c2, s, st.ri);
     st.u = (VAR && a.av.energy_split) ? a.us[s] : R(0);
     double L = a.c.box_L[a.c.boxid[s]];
     st.L = (R)L;
@@ -391,11 +405,17 @@ template <class R, bool VAR = false> struct PassC2 {
   __device__ static void pair_s(const Args& a, State& st, const R* rj, const R*, uint32_t j,
                                 uint32_t) {
     if (a.c.spec && (st.ri[RC::C2_FLAG] > R(1.5) || rj[RC::C2_FLAG] > R(1.5))) return;  // winds
-    PairC2<R> p;
-    p.template forward<VAR>(st.ri, rj, st.L, st.halfL, a.av);
+    R d[3];
+    separation(st.ri, rj, st.L, st.halfL, d);
+    const R r2 = dot3(d, d);
+    R F[3];
+    PairC2<R>::template force<VAR>(st.ri, rj, d, r2, a.av, F);
 #pragma unroll
-    for (int k = 0; k < 3; ++k) st.a[k] += p.F[k];
-    const R E = p.work();
+    for (int p = 0; p < 3; ++p) st.a[p] += F[p];
+    const R* vi = st.ri + RC::C2_VEL;
+    const R* vj = rj + RC::C2_VEL;
+    // pair work E_ij = F.(v_j - v_i), formed identically from both sides
+    const R E = -(F[0] * (vi[0] - vj[0]) + F[1] * (vi[1] - vj[1]) + F[2] * (vi[2] - vj[2]));
     const R f = (VAR && a.av.energy_split) ? energy_share(true, E, st.u, a.us[j]) : R(0.5);
     st.e.add(f * E);
   }
@@ -611,20 +631,31 @@ __global__ void k_pack_state_c2(const uint8_t* __restrict__ flg, const int32_t* 
   if (s >= n || (flg[s] & 1)) return;
   using RC = Rec<R>;
   const int64_t p = perm[s];
-  R x[RC::XW];
-  get_x(xs, n, s, x);
+  R r[RC::C2];
+#pragma unroll
+  for (int k = 0; k < RC::C2; ++k) r[k] = R(0);
+  get_x(xs, n, s, r);
   const R rho = rho_state[p], u = us[s];
   const R cs = sqrt_(ggm1 * u);
-  R gv[9], vel[3], C[16], r[RC::C2];
+  R gv[9];
 #pragma unroll
   for (int k = 0; k < 9; ++k) gv[k] = gv_state[k * n + p];
-#pragma unroll
-  for (int k = 0; k < 3; ++k) vel[k] = v[k * n + p];
-  load_rec<16>(coef, s, C);
   const R div = gv[0] + gv[4] + gv[8];
   const bool flag = relax_dt > R(0) && exp_(fabs(div) * relax_dt) > R(8);
-  make_rates_record<R>(r, x, C, gv, R(1) / hs[s], vel, Vs[s], gm1 * rho * u, Cl * rho * cs,
-                       Cq * rho, flag ? R(1) : R(0));
+  r[RC::C2_IH] = R(1) / hs[s];
+  r[RC::C2_V] = Vs[s];
+  r[RC::C2_P] = gm1 * rho * u;
+  r[RC::C2_QA] = Cl * rho * cs;
+  r[RC::C2_QB] = Cq * rho;
+  r[RC::C2_FLAG] = flag ? R(1) : R(0);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) r[RC::C2_VEL + k] = v[k * n + p];
+  R C[16];
+  load_rec<16>(coef, s, C);
+#pragma unroll
+  for (int k = 0; k < 16; ++k) r[RC::C2_A + k] = C[k];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) r[RC::C2_GV + k] = gv[k];
   store_rec<RC::C2>(rec_c2, s, r);
   rhos[s] = rho;
 }

@@ -52,8 +52,8 @@ __global__ void k_hdot(int64_t n, const int32_t* __restrict__ perm, const R* __r
   const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (s >= n) return;
   using RC = Rec<R>;
-  const R* r = rec_c2 + s * RC::C2;
-  const R div_r = add_rn(add_rn(r[c2_gv(0, 0)], r[c2_gv(1, 1)]), r[c2_gv(2, 2)]);
+  const R* gv = rec_c2 + s * RC::C2 + RC::C2_GV;
+  const R div_r = add_rn(add_rn(gv[0], gv[4]), gv[8]);
   const double div = (double)div_r;
   const double h = (double)hs[s];
   const double dn = div_rn(mul_rn(n_h, cbrt((double)Vs[s])), h);   // Delta_N

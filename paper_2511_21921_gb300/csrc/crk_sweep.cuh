@@ -563,15 +563,14 @@ __device__ __forceinline__ void rk_gradient(const R* C, const R* x, R W, R g, bo
 
 // viscosity constants, converted once to the working precision
 template <class R> struct AVParams {
-  R eta_crit, inv_fold, eps2;
+  R eta_crit, eta_fold, eps2;
   int limiter;
-  int relax;         // relaxation flags can be set (relax_dt > 0)
   int q_side;        // each side's viscosity with its own gradient
   int energy_split;  // pair work shared by the specific energies
 };
 template <class R> AVParams<R> make_av(const crk_params& p) {
-  return AVParams<R>{(R)p.eta_crit, (R)(1.0 / p.eta_fold), (R)p.eps2, p.limiter,
-                     p.relax_dt > 0.0 ? 1 : 0, p.q_side, p.energy_split};
+  return AVParams<R>{(R)p.eta_crit, (R)p.eta_fold, (R)p.eps2, p.limiter, p.q_side,
+                     p.energy_split};
 }
 
 // Share f_ij of the pair work E_ij that particle i receives (compatible energy,
@@ -587,192 +586,78 @@ __device__ __forceinline__ R energy_share(bool split, R E, R ui, R uj) {
   return R(0.5) * (R(1) + (E > R(0) ? q : -q));
 }
 
-// Rate record (Rec::C2) of one particle from its coefficients C (A, B, grad A,
-// grad B), velocity gradient gv (row major) and the rest.
-template <class R>
-__device__ __forceinline__ void make_rates_record(R* r, const R* x, const R* C, const R* gv, R ih,
-                                                  const R* v, R V, R P, R qa, R qb, R flag) {
-  using RC = Rec<R>;
-#pragma unroll
-  for (int k = 0; k < RC::C2; ++k) r[k] = R(0);
-  const R A = C[0];
-  R* M = r + RC::C2_M;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    M[k] = fma_(A, C[1 + k], C[4 + k]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a)
-      M[4 + 4 * a + k] = fma_(A, C[7 + 3 * k + a], C[4 + k] * C[1 + a]);
-    M[4 + 4 * k + 3] = A * C[1 + k];
-  }
-  M[3] = A;
-#pragma unroll
-  for (int p = 0; p < 3; ++p)
-#pragma unroll
-    for (int q = 0; q < 3; ++q) r[c2_gv(p, q)] = gv[3 * p + q];
-  r[RC::C2_IH] = ih;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) r[RC::C2_VEL + k] = v[k];
-  r[RC::C2_V] = V;
-  r[RC::C2_P] = P;
-  r[RC::C2_QA] = -qa;
-  r[RC::C2_QB] = qb;
-  r[RC::C2_FLAG] = flag;
-#pragma unroll
-  for (int k = 0; k < RC::XW; ++k) r[RC::C2_X + k] = x[k];
-}
-
-// The particle's own rate record for the pair loop: the pair arithmetic works
-// in e = x_j - x_i for both members, so the own side's columns (which multiply
-// x_i - x_j) are negated once here.
-template <class R>
-__device__ __forceinline__ void load_own_rates_record(const R* __restrict__ rec, int64_t s, R* ri) {
-  load_rec<Rec<R>::C2>(rec, s, ri);
-#pragma unroll
-  for (int k = 4; k < 16; ++k) ri[Rec<R>::C2_M + k] = -ri[Rec<R>::C2_M + k];
-}
-
-// Forward part of one pair, shared by the rate sweep and its adjoint: force
-// F_ij = m_i a_ij and the quantities the reverse needs.  Where both members go
-// through the same scalar formula the two are one packed pair (i, j); the
-// 4-vectors (u, lin) = M (1, e) are packed along the vector.  Every operand
-// that both members' threads form comes out of the same expression on both
-// sides, so F_ji = -F_ij bit for bit.  pa and pb, on whose sum the limiter's
-// derivative is ill conditioned (1/(pa+pb)^2 where both nearly vanish), are
-// formed from the whole velocity gradients in a fixed order of fused
-// multiply-adds, the one the compiler gives x0 y0 + x1 y1 + x2 y2.
+// The shared pair kernel: returns F (force on i from j, = m_i a_ij) and the
+// intermediate quantities the adjoint needs.  xi/xj are the full c2 records.
 template <class R> struct PairC2 {
   using RC = Rec<R>;
-  using D2 = P2<R>;
-  R e[3], r2, r, ir;
-  D2 e0, e1, e2, e01;                // (e_a, e_a) and (e_0, e_1)
-  D2 ih, ih2, W, g, om4;             // (i, j)
-  D2 ui01, ui2l, uj01, uj2l;         // (u_0, u_1), (u_2, lin) of i and of j
-  R gli, glj;                        // g lin
-  R Gi[3], Gj[3], dG[3];
-  R gie[3], gje[3], pa, pb;          // grad v e, e.grad v e
-  R is, phi0, damp, phi, z, ihmin;  // is: 1/(pa + pb), 0 where they differ in sign
-  R vij[3], vx;
-  D2 iD, hD, t, mu, qs;              // 1/D, ih/D, mu before the clamp, mu, QB mu - QA
-  R ViVj, Pi, VV, PP, Qi, Qj, F[3];
-
-  __device__ static __forceinline__ void column(const R* rec, D2& c01, D2& c2l, const D2* ea) {
-    const R* M = rec + RC::C2_M;
-    c01 = mk2(M[0], M[1]);
-    c2l = mk2(M[2], M[3]);
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      c01 = fma2(mk2(M[4 + 4 * a], M[5 + 4 * a]), ea[a], c01);
-      c2l = fma2(mk2(M[6 + 4 * a], M[7 + 4 * a]), ea[a], c2l);
-    }
+  // limiter phi from a = x.gv_i.x, b = x.gv_j.x:  4ab/(a+b)^2 when ab > 0
+  __device__ static __forceinline__ R limiter_phi(R a, R b) {
+    const R ab = a * b;
+    if (!(ab > R(0))) return R(0);
+    const R sm = a + b;
+    return R(4) * ab / (sm * sm);
   }
-  // o = grad v e; row by row fma(g_2, e_2, fma(g_0, e_0, g_1 e_1))
-  __device__ static __forceinline__ void gradv_e(const R* rec, const R* e, const D2* ea, R* o) {
-    const R* G = rec + RC::C2_GV;
-    const D2 t = fma2(mk2(G[4], G[5]), ea[2],
-                      fma2(mk2(G[0], G[1]), ea[0], mul2(mk2(G[2], G[3]), ea[1])));
-    get2(t, o[0], o[1]);
-    o[2] = fma_(G[8], e[2], fma_(G[6], e[0], rmul(G[7], e[1])));
-  }
-
-  template <bool VAR>
-  __device__ __forceinline__ void forward(const R* ri, const R* rj, R L, R halfL,
-                                          const AVParams<R>& av) {
-    separation(rj + RC::C2_X, ri + RC::C2_X, L, halfL, e);
-    r2 = dot3(e, e);
-    ir = r2 > R(0) ? rsqrt_(r2) : R(0);
-    r = r2 * ir;
-    const D2 ea[3] = {dup2(e[0]), dup2(e[1]), dup2(e[2])};
-    e0 = ea[0];
-    e1 = ea[1];
-    e2 = ea[2];
-    e01 = mk2(e[0], e[1]);
-    // Wendland C4 of both members (see wendland())
-    ih = mk2(ri[RC::C2_IH], rj[RC::C2_IH]);
-    const D2 q = mul2(dup2(r), ih);
-    R oa, ob;
-    get2(fma2(q, dup2(R(-1)), dup2(R(1))), oa, ob);
-    const D2 om = mk2(oa > R(0) ? oa : R(0), ob > R(0) ? ob : R(0));
-    const D2 om2 = mul2(om, om);
-    om4 = mul2(om2, om2);
-    ih2 = mul2(ih, ih);
-    const D2 ih3 = mul2(ih2, ih);
-    constexpr R cw = R(Wend<R>::cw), cg = R(Wend<R>::cg);
-    W = mul2(mul2(ih3, mul2(om4, om2)),
-             fma2(q, fma2(q, dup2(R(35.0 / 3.0) * cw), dup2(R(6) * cw)), dup2(cw)));
-    g = mul2(mul2(mul2(ih3, ih2), mul2(om4, om)), fma2(q, dup2(R(5) * cg), dup2(cg)));
-    // corrected gradients
-    column(ri, ui01, ui2l, ea);
-    column(rj, uj01, uj2l, ea);
-    if (av.relax && !(ri[RC::C2_FLAG] == R(0) && rj[RC::C2_FLAG] == R(0))) {
-      // uncorrected kernel: u = 0, lin = 1
-      ui01 = uj01 = dup2(R(0));
-      ui2l = uj2l = mk2(R(0), R(1));
-    }
-    R Wi, Wj, gi, gj;
-    get2(W, Wi, Wj);
-    get2(g, gi, gj);
-    gli = gi * hi2(ui2l);
-    glj = gj * hi2(uj2l);
-    get2(fma2(dup2(-gli), e01, mul2(dup2(Wi), ui01)), Gi[0], Gi[1]);
-    Gi[2] = fma_(-gli, e[2], rmul(Wi, lo2(ui2l)));
-    get2(fma2(dup2(glj), e01, mul2(dup2(Wj), uj01)), Gj[0], Gj[1]);
-    Gj[2] = fma_(glj, e[2], rmul(Wj, lo2(uj2l)));
+  template <bool VAR = false>
+  __device__ static __forceinline__ void force(const R* ri, const R* rj, const R* d, R r2,
+                                               const AVParams<R>& av, R* F) {
+    const R r = radius(r2);
+    const bool rk = ri[RC::C2_FLAG] == R(0) && rj[RC::C2_FLAG] == R(0);
+    R Wi, gi, Wj, gj;
+    wendland(r, ri[RC::C2_IH], Wi, gi);
+    wendland(r, rj[RC::C2_IH], Wj, gj);
+    const R nd[3] = {-d[0], -d[1], -d[2]};
+    R Gi[3], Gj[3];
+    rk_gradient(ri + RC::C2_A, d, Wi, gi, rk, Gi);
+    rk_gradient(rj + RC::C2_A, nd, Wj, gj, rk, Gj);
+    // artificial viscosity
+    const R* gvi = ri + RC::C2_GV;
+    const R* gvj = rj + RC::C2_GV;
+    R gix[3], gjx[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) dG[k] = rsub(Gi[k], Gj[k]);
-    // limited relative velocity
-    gradv_e(ri, e, ea, gie);
-    gradv_e(rj, e, ea, gje);
-    pa = fma_(e[2], gie[2], fma_(e[0], gie[0], rmul(e[1], gie[1])));
-    pb = fma_(e[2], gje[2], fma_(e[0], gje[0], rmul(e[1], gje[1])));
-    phi = phi0 = is = R(0);
-    damp = R(1);
-    z = R(0);
-    ihmin = fmin(ri[RC::C2_IH], rj[RC::C2_IH]);
+    for (int p = 0; p < 3; ++p) {
+      gix[p] = gvi[3 * p] * d[0] + gvi[3 * p + 1] * d[1] + gvi[3 * p + 2] * d[2];
+      gjx[p] = gvj[3 * p] * d[0] + gvj[3 * p + 1] * d[1] + gvj[3 * p + 2] * d[2];
+    }
+    R phi = R(0);
+    const R ihi = ri[RC::C2_IH], ihj = rj[RC::C2_IH];
     if (av.limiter) {
-      // phi = 4 pa pb / (pa + pb)^2 where both have one sign; damped below eta_crit
-      is = pa * pb > R(0) ? rcp_(pa + pb) : R(0);
-      phi0 = (R(4) * (pa * is)) * (pb * is);
-      z = (r * ihmin - av.eta_crit) * av.inv_fold;
-      z = z < R(0) ? z : R(0);
-      damp = gauss_(z);
-      phi = phi0 * damp;
+      const R pa = d[0] * gix[0] + d[1] * gix[1] + d[2] * gix[2];
+      const R pb = d[0] * gjx[0] + d[1] * gjx[1] + d[2] * gjx[2];
+      phi = limiter_phi(pa, pb);
+      const R eta = r * fmin(ihi, ihj);
+      if (eta < av.eta_crit) {
+        const R z = (eta - av.eta_crit) / av.eta_fold;
+        phi = phi * exp_(-(z * z));
+      }
     }
+    const R hphi = R(0.5) * phi;
+    R vh[3];
 #pragma unroll
-    for (int k = 0; k < 3; ++k) vij[k] = ri[RC::C2_VEL + k] - rj[RC::C2_VEL + k];
-    const R ve = fma_(vij[2], e[2], fma_(vij[0], e[0], rmul(vij[1], e[1])));
-    vx = -fma_(R(0.5) * phi, pa + pb, ve);
-    // artificial viscosity of both members
-    const D2 Dd = fma2(dup2(r2), ih2, dup2(av.eps2));
-    iD = mk2(rcp_(lo2(Dd)), rcp_(hi2(Dd)));
-    hD = mul2(ih, iD);
-    t = mul2(dup2(vx), hD);
-    R ta, tb;
-    get2(t, ta, tb);
-    mu = mk2(ta < R(0) ? ta : R(0), tb < R(0) ? tb : R(0));
-    qs = fma2(mk2(ri[RC::C2_QB], rj[RC::C2_QB]), mu, mk2(ri[RC::C2_QA], rj[RC::C2_QA]));
-    get2(mul2(mu, qs), Qi, Qj);
-    ViVj = rmul(ri[RC::C2_V], rj[RC::C2_V]);
-    PP = radd(ri[RC::C2_P], rj[RC::C2_P]);
-    VV = R(-0.5) * ViVj;
+    for (int p = 0; p < 3; ++p)
+      vh[p] = (ri[RC::C2_VEL + p] - rj[RC::C2_VEL + p]) - hphi * (gix[p] + gjx[p]);
+    const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
+    R mui = vx * ihi / (r2 * (ihi * ihi) + av.eps2);
+    R muj = vx * ihj / (r2 * (ihj * ihj) + av.eps2);
+    mui = mui < R(0) ? mui : R(0);
+    muj = muj < R(0) ? muj : R(0);
+    const R Qi = mui * (ri[RC::C2_QB] * mui - ri[RC::C2_QA]);
+    const R Qj = muj * (rj[RC::C2_QB] * muj - rj[RC::C2_QA]);
     if (VAR && av.q_side) {
       // (P_i + P_j)(G_ij - G_ji) + 2 (Q_ij G_ij - Q_ji G_ji), the two products
       // rounded on their own so that the j side forms exactly the negation
+      const R VV = R(-0.5) * (ri[RC::C2_V] * rj[RC::C2_V]);
+      const R PP = ri[RC::C2_P] + rj[RC::C2_P];
 #pragma unroll
       for (int p = 0; p < 3; ++p) {
         const R qg = rsub(rmul(Qi, Gi[p]), rmul(Qj, Gj[p]));
-        F[p] = VV * radd(rmul(PP, dG[p]), R(2) * qg);
+        F[p] = VV * radd(rmul(PP, Gi[p] - Gj[p]), R(2) * qg);
       }
-      Pi = R(0);
-    } else {
-      Pi = radd(PP, radd(Qi, Qj));
-#pragma unroll
-      for (int p = 0; p < 3; ++p) F[p] = rmul(rmul(VV, Pi), dG[p]);
+      return;
     }
-  }
-  // pair work E_ij = F.(v_j - v_i), formed identically from both sides
-  __device__ __forceinline__ R work() const {
-    return -fma_(F[2], vij[2], fma_(F[0], vij[0], rmul(F[1], vij[1])));
+    const R Pi = (ri[RC::C2_P] + rj[RC::C2_P]) + (Qi + Qj);
+    const R pre = R(-0.5) * (ri[RC::C2_V] * rj[RC::C2_V]) * Pi;
+#pragma unroll
+    for (int p = 0; p < 3; ++p) F[p] = pre * (Gi[p] - Gj[p]);
   }
 };
 
