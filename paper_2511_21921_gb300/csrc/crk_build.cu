@@ -922,21 +922,30 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
   // a column that overflowed is left empty: its later slots were not written
   const int cg = need <= cap_pp ? kg : 0;
   const int cs = need <= cap_pp ? ks : 0;
-  // close the gap: move scatter-only entries from the back of the column to
-  // just behind the gather part, so that a union list is slots 0 .. cg + cs - 1
-  // (only the entries beyond the final end move, into slots no entry holds)
+  // close the gap: scatter-only entry t moves from slot cap_pp - 1 - t to
+  // cg + t, so that a union list is slots 0 .. cg + cs - 1 in the order found
   {
     const int gap = (int)cap_pp - cg - cs;
-    const int mv = cs < gap ? cs : gap;
     uint32_t* c0 = ell + wbase;
-    for (int t = 0; t < mv; t += 4) {
-      uint32_t e[4];
+    if (cs <= gap) {
+      for (int t = 0; t < cs; t += 4) {
+        uint32_t e[4];
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        e[q] = t + q < mv ? c0[(cap_pp - 1 - t - q) * 32] : 0u;
+        for (int q = 0; q < 4; ++q)
+          e[q] = t + q < cs ? c0[(cap_pp - 1 - t - q) * 32] : 0u;
 #pragma unroll
-      for (int q = 0; q < 4; ++q)
-        if (t + q < mv) c0[(int64_t)(cg + t + q) * 32] = e[q];
+        for (int q = 0; q < 4; ++q)
+          if (t + q < cs) c0[(int64_t)(cg + t + q) * 32] = e[q];
+      }
+    } else if (cs > 0) {
+      // a nearly full column: the two ranges overlap; reverse, then shift down
+      uint32_t* r0 = c0 + (cap_pp - cs) * 32;
+      for (int t = 0; t < cs / 2; ++t) {
+        const uint32_t x = r0[(int64_t)t * 32], y = r0[(int64_t)(cs - 1 - t) * 32];
+        r0[(int64_t)t * 32] = y;
+        r0[(int64_t)(cs - 1 - t) * 32] = x;
+      }
+      for (int t = 0; gap > 0 && t < cs; ++t) c0[(int64_t)(cg + t) * 32] = r0[(int64_t)t * 32];
     }
   }
   if (live) {
