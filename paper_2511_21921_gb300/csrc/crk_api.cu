@@ -573,7 +573,9 @@ crk_status crk_autotune(crk_plan* plan, crk_stream_t stream, void* ws, const voi
     int best = 0;
     for (int k = 1; k < CRK_TUNE_VARIANTS; ++k)
       if (tsum[q][k] > 0 && tsum[q][k] < tsum[q][best]) best = k;
-    if (s != CRK_OK || (q >= 4 && !adj)) best = 0;
+    // a sweep that was not timed keeps the rule's variant
+    if (s != CRK_OK || (q >= 4 && !adj))
+      best = default_variant(queues[q], P.p.precision, P.ly.n);
     P.variant[queues[q]] = best;
     if (choice_out) choice_out[q] = best;
     if (ms_out)

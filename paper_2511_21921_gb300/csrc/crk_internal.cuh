@@ -34,7 +34,11 @@ struct Plan {
   int64_t n = 0;
   int32_t nb = 0;
   Tuning tune[16];
-  int variant[16] = {};  // launch variant per sweep: v % 3 -> MB0..MB2, v / 3 -> load mode
+  // launch variant per sweep: v % 3 -> MB0..MB2, v / 3 -> load mode; kAutoVariant
+  // until the autotuner or crk_tune_set chose one (default_variant then)
+  static constexpr int kAutoVariant = -1;
+  int variant[16];
+  Plan() { std::fill(variant, variant + 16, kAutoVariant); }
   // instrumentation
   long long launches = 0;
   bool timing = false;
@@ -69,6 +73,35 @@ int scan_launches(int64_t n);  // kernels exclusive_scan launches for n elements
 constexpr int kLptItemsPerWarp = 8;
 inline bool lpt_worthwhile(int64_t items, int64_t warps) {
   return items <= (int64_t)kLptItemsPerWarp * warps;
+}
+
+// Launch variant of a sweep on n particles when none was chosen.  Mixed form,
+// milliseconds on one GB300 of plain loads (variant 0) against the variant
+// taken, lognormal boxes of variance 1.5, at 16 k / 60 k / 262 k / 2.1 M particles:
+//   volume    0.052/0.066/0.160/1.00 -> ring 0.039/0.061, deep buffers 0.107/0.63
+//   moments   0.063/0.079/0.327/2.17 -> ring 0.051/0.068, warp ring 0.200/1.32
+//   density   0.059/0.079/0.321/2.11 -> deep buffers 0.047/0.061/0.211/1.40
+//   rates     0.121/0.193/0.600/4.17 -> warp ring 0.100/0.156/0.516/3.74
+//   adjoint   rates 0.185/0.310/1.27/9.30 -> double buffer 0.160/0.266/0.966/7.46
+//             density 0.105/0.222/0.641/4.53 -> 0.074/0.174/0.581/4.26
+//             moments 0.102/0.172/0.598/4.14 -> 0.070/0.163/0.566/4.14
+//             volume 0.072/0.091/0.208/1.36 -> 0.047/0.065/0.160/1.24
+// Small boxes have about one warp per scheduler: there the ring hides most of
+// the gather latency, and more registers cost nothing.  The deep buffers with
+// their register cap need enough warps to fill the SMs (from about 50 k
+// particles for the volume sweep, where 0.0475 at 60 k meets the ring's 0.061),
+// the capped warp ring of the moment sweep from about 100 k (0.120 at 120 k
+// against 0.124).  All of them give the same bits.  The FP64 form is bound by
+// its pipe: every variant is within 5 % of plain loads.
+inline int default_variant(int queue, int precision, int64_t n) {
+  if (precision == CRK_FP64) return 0;
+  switch (queue) {
+    case Q_B1: return n < 50000 ? 3 : 14;
+    case Q_B2: return n < 100000 ? 3 : 17;
+    case Q_C1: return 12;
+    case Q_C2: return 9;
+    default: return 6;
+  }
 }
 
 template <class R>
