@@ -9,6 +9,8 @@
 // the tree is a linear BVH over Morton-ordered buckets (one CUDA thread per
 // node, no spin waits), and its only job is to produce neighbor lists that
 // every later sweep reads without further distance tests.
+#include <type_traits>
+
 #include "crk_internal.cuh"
 
 namespace crk {
@@ -483,39 +485,26 @@ __device__ __forceinline__ void ld8(const float* p, float* o) {
 // ---------------------------------------------------------------------------
 // neighbor lists: one thread per sorted particle traverses the tree
 // ---------------------------------------------------------------------------
-template <class R> struct XI;
-template <> struct XI<float> { float v[6]; };
-template <> struct XI<double> { double v[3]; };
-
-__device__ __forceinline__ void load_x(const float* xs, int64_t n, int64_t s, float* o) {
-#pragma unroll
-  for (int a = 0; a < 6; ++a) o[a] = xs[a * n + s];
-}
-__device__ __forceinline__ void load_x(const double* xs, int64_t n, int64_t s, double* o) {
-#pragma unroll
-  for (int a = 0; a < 3; ++a) o[a] = xs[a * n + s];
-}
-// r^2 as in the oracle for double (no contraction); plain float otherwise
+// r^2 as the definition forms it (no contraction)
 __device__ __forceinline__ double norm2(const double* d) {
   return __dadd_rn(__dadd_rn(__dmul_rn(d[0], d[0]), __dmul_rn(d[1], d[1])), __dmul_rn(d[2], d[2]));
 }
-__device__ __forceinline__ float norm2(const float* d) {
-  return fmaf(d[2], d[2], fmaf(d[1], d[1], d[0] * d[0]));
-}
 __device__ __forceinline__ double sq(double a) { return __dmul_rn(a, a); }
-__device__ __forceinline__ float sq(float a) { return a * a; }
 
-// Exact pair predicate of the mixed form.  The float candidate test works on
-// positions rounded to float (and, for the nearest-image staging, shifted by a
-// float L), so r^2 carries an error of at most 2^-24 (10 sqrt(3) L r + 6 r^2)
-// against the double r^2 of the caller's positions (each coordinate within
-// 5 * 2^-24 L of its exact image difference, three roundings in the sum of
-// squares, one in h^2).  A decision r^2 < h^2 is therefore certain outside the
-// band |r^2 - h^2| <= tol(h) below (wider by a third in the L term and more in
-// the h^2 term); inside it the pair is decided again in double exactly as the
+// Exact pair predicate.  The float candidate test of both forms works on
+// positions rounded to float (and shifted by a float L to an image), so r^2
+// carries an error of at most 2^-24 (10 sqrt(3) L r + 6 r^2) against the double
+// r^2 of the caller's positions (each coordinate within 5 * 2^-24 L of its exact
+// image difference, three roundings in the sum of squares), and a float h^2 of
+// at most 3 * 2^-24 h^2 (one rounding, and in the FP64 form h rounded to
+// float).  A decision r^2 < h^2 is therefore certain outside the band
+// |r^2 - h^2| <= tol(h) below (wider by a third in the L term and more in the
+// h^2 term); inside it the pair is decided again in double exactly as the
 // definition states -- minimum image decided and formed in double, r^2 summed
-// without contraction, compared with the squared (float) smoothing lengths --
-// so the mixed lists equal the FP64 lists of the same inputs.
+// without contraction, compared with the squared smoothing lengths -- so the
+// lists of both forms are those of the double predicate.  (Testing every
+// candidate of the FP64 form in double took 2.89 ms of its build on 13,824
+// particles: GB300 runs FP64 at 1/64 of the FP32 rate.)
 __device__ __forceinline__ float list_band(float h, float L) {
   return 5.9604645e-8f * fmaf(16.f * h, h, 24.f * L * h);
 }
@@ -527,17 +516,12 @@ __device__ __forceinline__ double exact_r2(const double* __restrict__ xd, int64_
   separation(a, b, L, 0.5 * L, d);
   return norm2(d);
 }
-// 1: certainly inside (r^2 < h^2), 0: certainly outside, -1: within the band
-__device__ __forceinline__ int band_decide(float r2, float h2, float tol) {
-  return r2 < h2 - tol ? 1 : (r2 > h2 + tol ? 0 : -1);
-}
-
 // One warp per 32 consecutive sorted particles walks the tree once for the
 // whole group (separately for each box present in the group): nodes are
 // tested 32 at a time against the group's bounding box grown by
 // max(h over the group, h_max of the node); overlapping buckets are staged
 // 4 at a time (32 particles) in shared memory and every lane tests its own
-// particle against all 32 with the exact pair predicate.  Traversal order is
+// particle against all 32.  Traversal order is
 // fixed, so the counting and the filling pass see the same entries.
 // Center, half extent and largest h of the lanes with `in` set (all lanes
 // take part in the shuffles).
@@ -567,28 +551,37 @@ __device__ __forceinline__ void group_bounds(bool in, const float* p, float h, f
 }
 
 constexpr int kNbrWarps = 4;
-constexpr int kNodeStack = 2048;
+// Resident blocks per SM (80 registers a thread, 16 KB of shared memory a block).
+// The build is bound by issue (60 % active): a third of its time is the tree
+// walk and the staging of candidates, a fifth the 32-candidate tests, a quarter
+// the emission of hits.  262,144 / 2.1 M / 16.8 M particles: 0.685 / 4.5 / 33.8 ms
+// with distances and bands evaluated again per hit, 0.558 / 3.68 / 27.0 ms with
+// the masks; 5 blocks 0.572 / 3.97 / 29.5, 8 blocks (64 registers) 0.590 / 3.66 /
+// 26.4.
+constexpr int kNbrBlocks = 6;
+// Node stack of a warp.  Taking 32 nodes a step adds at most 32 to it; from
+// three quarters on the walk takes one node a step, which adds at most one per
+// level of the tree (94 at most: 64 key bits and 30 index bits), so it cannot
+// overflow.  (The deepest seen with 32 a step: 268, the clumpy 128^3 box.)
+constexpr int kNodeStack = 512;
 
 template <class R>
-__global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
-    const uint64_t* __restrict__ keys, const R* __restrict__ xs, const R* __restrict__ hs,
-    const int32_t* __restrict__ boxid,
+__global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
+    const uint64_t* __restrict__ keys, const R* __restrict__ hs, const int32_t* __restrict__ boxid,
     const double* __restrict__ box_L, int64_t n, int64_t nbk, int64_t ni, int64_t nt,
     const float* __restrict__ nrec, const float4* __restrict__ p4, int32_t* __restrict__ cnt_g, int32_t* __restrict__ cnt_s, int32_t* __restrict__ wlen_g,
     int32_t* __restrict__ wlen_s, uint32_t* __restrict__ ell, int64_t cap_pp, DevHeader* hdr,
     const double* __restrict__ xd, const int32_t* __restrict__ perm,
     const float* __restrict__ hbox) {
-  constexpr int XW = Prec<R>::XW;
-  constexpr bool MIXED = sizeof(R) == 4;
   __shared__ int32_t stk[kNbrWarps][kNodeStack];
   __shared__ int32_t cand[kNbrWarps][64];
-  __shared__ R sx[kNbrWarps][XW][32];
-  __shared__ R sh[kNbrWarps][32];
-  // staged candidates: nearest-image float position and h^2 widened by the
-  // rounding band (the union mask), then h^2 and the band itself
-  __shared__ float4 s4[kNbrWarps][64];
-  __shared__ float2 sb[kNbrWarps][64];
+  // staged candidates, one array per component so that four (a 128-bit load)
+  // arrive at once: float position (of the nearest image, where one serves the
+  // whole group), h^2, its rounding band, index; and the slot of each lane's own
+  // particle (-1: not staged)
+  __shared__ float4 stage[kNbrWarps][5][16];
   __shared__ int32_t sj[kNbrWarps][64];
+  __shared__ int32_t self_at[kNbrWarps][32];
   const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t w = (int64_t)blockIdx.x * kNbrWarps + wib;
   const int64_t nw = (n + 31) / 32;
@@ -596,26 +589,22 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
   const uint32_t lt = (1u << lane) - 1u;
   const int64_t s = w * 32 + lane;
   const bool live = s < n;
-  R xi[XW];
-  R hi = R(0);
+  float hi = 0.f;
   int32_t bi = -1;
   float p[3] = {0.f, 0.f, 0.f};
   if (live) {
-    load_x(xs, n, s, xi);
-    hi = hs[s];
+    const float4 own = p4[s];
+    p[0] = own.x;
+    p[1] = own.y;
+    p[2] = own.z;
+    hi = own.w;
     bi = boxid[s];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) p[a] = (float)xpos(xs, n, s, a);
-  } else {
-#pragma unroll
-    for (int a = 0; a < XW; ++a) xi[a] = R(0);
   }
-  const R hi2 = sq(hi);
   // gather entries fill this lane's column from the front, scatter-only
   // entries from the back (moved up at the end); kg + ks > cap_pp means the
   // column overflowed
   int kg = 0, ks = 0;
-  const int64_t wbase = w * cap_pp * 32 + lane;
+  uint32_t* col = ell + w * cap_pp * 32 + lane;
   bool overflow = false;
   unsigned long long cnt_nodes = 0, cnt_buckets = 0;
   // Lane groups to traverse: one per box present in the warp, each split at
@@ -640,15 +629,14 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
     const int lead = __ffs(m) - 1;
     const int32_t b = __shfl_sync(kFull, bi, lead);
     const double Ld = box_L[b];
-    const R L = (R)Ld, halfL = (R)(0.5 * Ld);
     const float Lf = (float)Ld, halfLf = (float)(0.5 * Ld);
     float gc[3], ge[3], hg;
-    group_bounds(act, p, (float)hi, gc, ge, hg);
-    // nearest-image staging is exact for every pair in reach when the group
-    // extent plus the largest search radius stays below half the box
+    group_bounds(act, p, hi, gc, ge, hg);
+    // one image of a candidate, the one nearest the group's center, serves
+    // every pair in reach when the group extent plus the largest search radius
+    // stays below half the box; otherwise every pair wraps on its own
     const float reach = fmaxf(hg, __ldg(hbox + b));  // the largest h of the box
-    const bool fast = sizeof(R) == 4 &&
-                      2.f * fmaxf(ge[0], fmaxf(ge[1], ge[2])) + reach < 0.49f * Lf;
+    const bool one_image = 2.f * fmaxf(ge[0], fmaxf(ge[1], ge[2])) + reach < 0.49f * Lf;
     if (__popc(m) > 2 && ntodo <= 6) {
       const uint64_t lk = __shfl_sync(kFull, mykey, lead);
       uint64_t kx = act ? (mykey ^ lk) : 0ull;
@@ -659,8 +647,8 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
         const unsigned m1 = __ballot_sync(kFull, act && ((mykey >> P) & 1ull));
         const unsigned m0 = m & ~m1;
         float c0[3], e0[3], h0, c1[3], e1[3], h1;
-        group_bounds((m0 >> lane) & 1u, p, (float)hi, c0, e0, h0);
-        group_bounds((m1 >> lane) & 1u, p, (float)hi, c1, e1, h1);
+        group_bounds((m0 >> lane) & 1u, p, hi, c0, e0, h0);
+        group_bounds((m1 >> lane) & 1u, p, hi, c1, e1, h1);
         const float V = (2.f * ge[0] + 2.f * hg) * (2.f * ge[1] + 2.f * hg) * (2.f * ge[2] + 2.f * hg);
         const float V0 = (2.f * e0[0] + 2.f * h0) * (2.f * e0[1] + 2.f * h0) * (2.f * e0[2] + 2.f * h0);
         const float V1 = (2.f * e1[0] + 2.f * h1) * (2.f * e1[1] + 2.f * h1) * (2.f * e1[2] + 2.f * h1);
@@ -672,70 +660,96 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
       }
     }
     int sp = 0, nc = 0;
-    int ns = 0;  // candidates waiting in the stage (float path)
-    const float hi2f = (float)hi * (float)hi;
-    const float tol_i = list_band((float)hi, Lf);
-    const float hi2w = hi2f + tol_i;
-    // the exact predicate for a pair within the rounding band (mixed form)
-    auto exact_pair = [&](int32_t j, bool& g, bool& sc) {
-      const double r2d = exact_r2(xd, n, perm[s], perm[j], Ld);
-      const double hj = (double)hs[j];
-      g = r2d < sq((double)hi);
-      sc = r2d < sq(hj);
-    };
-    // float predicate on the nearest images: no per-pair wrap.  The 32
-    // staged candidates are tested branch-free into one bit mask of the union
-    // predicate r^2 < max(h_i^2, h_j^2), widened by the rounding band; only
-    // the hits (a few per stage) are then emitted, in candidate order, with the
-    // same r^2 recomputed to tell gather from scatter-only and the pairs
-    // within the band decided exactly.  The emit loop diverges (a warp runs
-    // it as often as its busiest lane has hits), so it takes two hits per
-    // iteration: their loads and decisions overlap and the loop runs about
-    // half as many times.
-    auto test_stage = [&]() {
-      uint32_t hit = 0u;
+    int ns = 0;  // candidates waiting in the stage
+    const float hi2f = hi * hi;
+    const float tol_i = list_band(hi, Lf);
+    const float iLf = 1.f / Lf;
+    // outside this range of box sides float squares could leave the float range:
+    // every pair is then decided exactly
+    const bool in_range = Lf > 1e-6f && Lf < 1e15f;
+    float* sx = reinterpret_cast<float*>(stage[wib]);  // component c, slot k: sx[64 c + k]
+    self_at[wib][lane] = -1;
+    // Tests the first 32 staged candidates (`filled` of them valid) against the
+    // lane's particle and appends the hits to its column.  Branch-free into
+    // three bit masks, two candidates per packed operation: gather
+    // (r^2 < h_i^2), scatter (r^2 < h_j^2) and, within the rounding band of
+    // either, uncertain; the sign bit of a difference is shifted into its mask.
+    // The few uncertain pairs are decided exactly; then only the hits are
+    // walked, each an index load and a store.  That walk diverges (a warp runs it
+    // as often as its busiest lane has hits), so nothing is evaluated in it: with
+    // the distance and both bands recomputed per hit it took two thirds of the
+    // build's instructions (442 million on 262,144 particles).  WRAP: minimum image
+    // per coordinate (the box length times the rounded quotient, subtracted).
+    auto test_stage = [&](int filled, auto wrap) {
+      using D2 = F2;
+      const D2 px = dup2(p[0]), py = dup2(p[1]), pz = dup2(p[2]);
+      const D2 minus = dup2(-1.f), nhi2 = dup2(-hi2f);
+      const D2 iL2 = dup2(iLf), nL2 = dup2(-Lf), mg = dup2(12582912.f), nmg = dup2(-12582912.f);
+      uint32_t G = 0u, S = 0u, X = 0u;
+      auto image = [&](D2 d) {
+        if constexpr (decltype(wrap)::value)
+          d = fma2(add2(fma2(d, iL2, mg), nmg), nL2, d);
+        return d;
+      };
 #pragma unroll
-      for (int k = 0; k < 32; ++k) {
-        const float4 t = s4[wib][k];
-        const float dx = p[0] - t.x, dy = p[1] - t.y, dz = p[2] - t.z;
-        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-        hit |= (r2 < fmaxf(hi2w, t.w) ? 1u : 0u) << k;
-      }
-      auto decide = [&](int k, int32_t& j, bool& g, bool& sc) {
-        j = sj[wib][k];
-        const float4 t = s4[wib][k];
-        const float2 hb = sb[wib][k];
-        const float dx = p[0] - t.x, dy = p[1] - t.y, dz = p[2] - t.z;
-        const float r2 = fmaf(dz, dz, fmaf(dy, dy, dx * dx));
-        const int gd = band_decide(r2, hi2f, tol_i);
-        const int sd = band_decide(r2, hb.x, hb.y);
-        g = gd == 1;
-        sc = sd == 1;
-        return gd < 0 || sd < 0;
-      };
-      auto emit = [&](int32_t j, bool g, bool sc) {
-        if (j == s || !(g || sc)) return;
-        const uint32_t e = (uint32_t)j | (g ? kGatherBit : 0u) | (sc ? kScatterBit : 0u);
-        if (kg + ks < cap_pp) {
-          const int64_t kk = g ? kg : cap_pp - 1 - ks;
-          ell[wbase + kk * 32] = e;
+      for (int q = 7; q >= 0; --q) {
+        const float4 tx = stage[wib][0][q], ty = stage[wib][1][q], tz = stage[wib][2][q];
+        const float4 th = stage[wib][3][q], tt = stage[wib][4][q];
+        const float* vx = &tx.x;
+        const float* vy = &ty.x;
+        const float* vz = &tz.x;
+        const float* vh = &th.x;
+        const float* vt = &tt.x;
+#pragma unroll
+        for (int u = 1; u >= 0; --u) {
+          const D2 dx = image(fma2(mk2(vx[2 * u], vx[2 * u + 1]), minus, px));
+          const D2 dy = image(fma2(mk2(vy[2 * u], vy[2 * u + 1]), minus, py));
+          const D2 dz = image(fma2(mk2(vz[2 * u], vz[2 * u + 1]), minus, pz));
+          const D2 r2 = fma2(dz, dz, fma2(dy, dy, mul2(dx, dx)));
+          float a[2], c[2];
+          get2(add2(r2, nhi2), a[0], a[1]);
+          get2(fma2(mk2(vh[2 * u], vh[2 * u + 1]), minus, r2), c[0], c[1]);
+#pragma unroll
+          for (int v = 1; v >= 0; --v) {
+            G = __funnelshift_l(__float_as_uint(a[v]), G, 1);
+            S = __funnelshift_l(__float_as_uint(c[v]), S, 1);
+            const float m = fminf(fabsf(a[v]) - tol_i, fabsf(c[v]) - vt[2 * u + v]);
+            X = __funnelshift_l(__float_as_uint(m), X, 1);
+          }
         }
-        if (g) ++kg; else ++ks;
-      };
-      while (hit) {
-        const int k1 = __ffs(hit) - 1;
-        hit &= hit - 1u;
-        const bool two = hit != 0u;
-        const int k2 = two ? __ffs(hit) - 1 : k1;
-        hit &= two ? hit - 1u : hit;
-        int32_t j1, j2;
-        bool g1, s1, g2, s2;
-        const bool x1 = decide(k1, j1, g1, s1);
-        const bool x2 = decide(k2, j2, g2, s2);
-        if (x1 && j1 != s) exact_pair(j1, g1, s1);
-        if (two && x2 && j2 != s) exact_pair(j2, g2, s2);
-        emit(j1, g1, s1);
-        if (two) emit(j2, g2, s2);
+      }
+      uint32_t valid = filled < 32 ? (1u << filled) - 1u : kFull;
+      const int own = self_at[wib][lane];
+      self_at[wib][lane] = own >= 32 ? own - 32 : -1;
+      if (own >= 0 && own < 32) valid &= ~(1u << own);
+      X = in_range ? X & valid : valid;
+      while (X) {
+        const int k = __ffs(X) - 1;
+        X &= X - 1u;
+        const int32_t j = sj[wib][k];
+        const double r2d = exact_r2(xd, n, perm[s], perm[j], Ld);
+        const uint32_t bit = 1u << k;
+        G = r2d < sq((double)hs[s]) ? G | bit : G & ~bit;
+        S = r2d < sq((double)hs[j]) ? S | bit : S & ~bit;
+      }
+      G &= valid;
+      S &= valid;
+      uint32_t U = G | S;
+      while (U) {
+        const int k = __ffs(U) - 1;
+        U &= U - 1u;
+        const uint32_t g = (G >> k) & 1u;
+        const uint32_t e = (uint32_t)sj[wib][k] | g << 31 | ((S >> k) & 1u) << 30;
+        const int at = g ? kg : (int)cap_pp - 1 - ks;
+        if (kg + ks < (int)cap_pp) col[at * 32] = e;
+        kg += (int)g;
+        ks += 1 - (int)g;
+      }
+    };
+    auto flush = [&](int filled) {
+      if (act) {
+        if (one_image) test_stage(filled, std::false_type{});
+        else test_stage(filled, std::true_type{});
       }
     };
     if (lane == 0) stk[wib][0] = (ni > 0) ? 0 : (int32_t)ni;
@@ -743,7 +757,8 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
     __syncwarp();
     while (sp > 0 || nc > 0) {
       if (sp > 0) {
-        const int take = sp < 32 ? sp : 32;
+        // one node at a time (depth first) once the stack is three quarters full
+        const int take = sp > kNodeStack * 3 / 4 ? 1 : (sp < 32 ? sp : 32);
         const int32_t node = lane < take ? stk[wib][sp - take + lane] : -1;
         sp -= take;
         cnt_nodes += take;
@@ -799,118 +814,66 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
         cnt_buckets += take;
         // stage the particles of buckets cand[nc .. nc+take)
         const int kb = lane >> 3;
-        if (fast) {
-          // float position moved to the periodic image nearest the group
-          // center (requested together with the box id).  A particle that
-          // lies farther from the group's box than max(h_group, h_j) cannot
-          // be a union neighbor of any lane and is dropped here; the others
-          // are appended to the stage, which is tested once it holds 32.
-          // Dropping preserves the order of the survivors, so every list
-          // comes out exactly as without the filter.
-          int64_t j = -1;
-          float4 t = make_float4(0.f, 0.f, 0.f, 0.f);
-          float2 tb = make_float2(0.f, 0.f);
-          bool pass = false;
-          if (kb < take) {
-            const int64_t jj = (int64_t)cand[wib][nc + kb] * kBucket + (lane & 7);
-            if (jj < n) {
-              const int32_t bj = __ldg(boxid + jj);
-              const float4 pj = __ldg(p4 + jj);
-              float q[3] = {pj.x, pj.y, pj.z};
-              const float hj = pj.w;
-              if (bj == b) {
-                j = jj;
-                float g2 = 0.f;
+        // A particle that lies farther from the group's box than
+        // max(h_group, h_j) cannot be a union neighbor of any lane and is
+        // dropped here; the others are appended to the stage, which is tested
+        // once it holds 32.  Dropping preserves the order of the survivors, so
+        // every list comes out exactly as without the filter.
+        int64_t j = -1;
+        float q[3] = {0.f, 0.f, 0.f}, hj = 0.f;
+        bool pass = false;
+        if (kb < take) {
+          const int64_t jj = (int64_t)cand[wib][nc + kb] * kBucket + (lane & 7);
+          if (jj < n) {
+            const int32_t bj = __ldg(boxid + jj);
+            const float4 pj = __ldg(p4 + jj);
+            q[0] = pj.x;
+            q[1] = pj.y;
+            q[2] = pj.z;
+            hj = pj.w;
+            if (bj == b) {
+              j = jj;
+              float g2 = 0.f;
 #pragma unroll
-                for (int a = 0; a < 3; ++a) {
-                  const float dd = gc[a] - q[a];
-                  q[a] += dd > halfLf ? Lf : (dd < -halfLf ? -Lf : 0.f);
-                  const float o = fabsf(q[a] - gc[a]) - ge[a];
-                  if (o > 0.f) g2 += o * o;
-                }
-                const float Rj = fmaxf(hg, hj) * 1.00001f + 1e-6f * Lf;
-                pass = g2 <= Rj * Rj;
-                tb = make_float2(hj * hj, list_band(hj, Lf));
-                t = make_float4(q[0], q[1], q[2], tb.x + tb.y);
+              for (int a = 0; a < 3; ++a) {
+                const float dd = gc[a] - q[a];
+                const float qn = q[a] + (dd > halfLf ? Lf : (dd < -halfLf ? -Lf : 0.f));
+                const float o = fabsf(qn - gc[a]) - ge[a];
+                if (o > 0.f) g2 += o * o;
+                if (one_image) q[a] = qn;
               }
+              const float Rj = fmaxf(hg, hj) * 1.00001f + 1e-6f * Lf;
+              pass = g2 <= Rj * Rj;
             }
           }
-          const unsigned mp = __ballot_sync(kFull, pass);
-          if (pass) {
-            const int at = ns + __popc(mp & lt);
-            s4[wib][at] = t;
-            sb[wib][at] = tb;
-            sj[wib][at] = (int32_t)j;
-          }
-          ns += __popc(mp);
+        }
+        const unsigned mp = __ballot_sync(kFull, pass);
+        if (pass) {
+          const int at = ns + __popc(mp & lt);
+#pragma unroll
+          for (int a = 0; a < 3; ++a) sx[64 * a + at] = q[a];
+          sx[192 + at] = hj * hj;
+          sx[256 + at] = list_band(hj, Lf);
+          sj[wib][at] = (int32_t)j;
+          if ((j >> 5) == w) self_at[wib][j & 31] = at;
+        }
+        ns += __popc(mp);
+        __syncwarp();
+        if (ns >= 32) {
+          flush(32);
           __syncwarp();
-          if (ns >= 32) {
-            if (act) test_stage();
-            __syncwarp();
-            if (lane < ns - 32) {
-              s4[wib][lane] = s4[wib][32 + lane];
-              sb[wib][lane] = sb[wib][32 + lane];
-              sj[wib][lane] = sj[wib][32 + lane];
-            }
-            ns -= 32;
-            __syncwarp();
-          }
-        } else {
-          int64_t j = -1;
-          if (kb < take) {
-            const int64_t jj = (int64_t)cand[wib][nc + kb] * kBucket + (lane & 7);
-            if (jj < n && boxid[jj] == b) j = jj;
-          }
-          sj[wib][lane] = (int32_t)j;
-          if (j >= 0) {
-            R t[XW];
-            load_x(xs, n, j, t);
+          if (lane < ns - 32) {
 #pragma unroll
-            for (int a = 0; a < XW; ++a) sx[wib][a][lane] = t[a];
-            sh[wib][lane] = hs[j];
+            for (int a = 0; a < 5; ++a) sx[64 * a + lane] = sx[64 * a + 32 + lane];
+            sj[wib][lane] = sj[wib][32 + lane];
           }
-          __syncwarp();
-          if (act) {
-            // exact predicate (the oracle's, for the FP64 form)
-#pragma unroll 4
-            for (int k = 0; k < 32; ++k) {
-              const int32_t j = sj[wib][k];
-              if (j < 0 || j == s) continue;
-              R xj[XW];
-#pragma unroll
-              for (int a = 0; a < XW; ++a) xj[a] = sx[wib][a][k];
-              R d[3];
-              separation(xi, xj, L, halfL, d);
-              const R r2 = norm2(d);
-              bool g = r2 < hi2;
-              bool sc = r2 < sq(sh[wib][k]);
-              if constexpr (MIXED) {
-                const float hj = (float)sh[wib][k];
-                const int gd = band_decide((float)r2, hi2f, tol_i);
-                const int sd = band_decide((float)r2, hj * hj, list_band(hj, Lf));
-                if (gd < 0 || sd < 0) exact_pair(j, g, sc);
-              }
-              if (!(g || sc)) continue;
-              const uint32_t e = (uint32_t)j | (g ? kGatherBit : 0u) | (sc ? kScatterBit : 0u);
-              if (kg + ks < cap_pp) {
-                const int64_t kk = g ? kg : cap_pp - 1 - ks;
-                ell[wbase + kk * 32] = e;
-              }
-              if (g) ++kg; else ++ks;
-            }
-          }
+          ns -= 32;
           __syncwarp();
         }
       }
     }
-    if (fast && ns > 0) {
-      // the last partial stage, padded with slots that never match
-      if (lane >= ns) {
-        s4[wib][lane] = make_float4(__int_as_float(0x7fffffff), 0.f, 0.f, __int_as_float(0x7fffffff));
-        sj[wib][lane] = -1;
-      }
-      __syncwarp();
-      if (act) test_stage();
+    if (ns > 0) {
+      flush(ns);  // the last partial stage
       __syncwarp();
       ns = 0;
     }
@@ -926,7 +889,7 @@ __global__ void __launch_bounds__(kNbrWarps * 32) k_nbr(
   // cg + t, so that a union list is slots 0 .. cg + cs - 1 in the order found
   {
     const int gap = (int)cap_pp - cg - cs;
-    uint32_t* c0 = ell + wbase;
+    uint32_t* c0 = col;
     if (cs <= gap) {
       for (int t = 0; t < cs; t += 4) {
         uint32_t e[4];
@@ -1202,7 +1165,7 @@ crk_status cell_build_impl(Plan* plan, cudaStream_t st, char* ws, int64_t n, int
   int32_t* wlen_s = reinterpret_cast<int32_t*>(ws + Ly.wlen_s);
   uint32_t* ell = reinterpret_cast<uint32_t*>(ws + Ly.ell);
   const unsigned gw = (unsigned)((Ly.nw + kNbrWarps - 1) / kNbrWarps);
-  k_nbr<R><<<gw, kNbrWarps * 32, 0, st>>>(k0, xs, hs, boxid, wbox, n, nbk, ni, nt, nrec, p4,
+  k_nbr<R><<<gw, kNbrWarps * 32, 0, st>>>(k0, hs, boxid, wbox, n, nbk, ni, nt, nrec, p4,
                                           cnt_g, cnt_s, wlen_g, wlen_s, ell, Ly.cap_pp, hdr, x,
                                           perm, reinterpret_cast<const float*>(hbox));
   int32_t* cost = reinterpret_cast<int32_t*>(ws + Ly.item_cost);

@@ -237,6 +237,40 @@ __device__ __forceinline__ double sqrt_(double x) { return sqrt(x); }
 __device__ __forceinline__ float exp_(float x) { return expf(x); }
 __device__ __forceinline__ double exp_(double x) { return exp(x); }
 
+// ---------------------------------------------------------------------------
+// Pairs of floats: one instruction (fma.rn.f32x2 and its relatives) works on
+// both halves, each rounding as the scalar operation does.  It takes one issue
+// slot instead of two for the same FP32 pipe time (measured on GB300: 75 TFLOP/s
+// of packed against 79 of scalar fused multiply-adds).
+// ---------------------------------------------------------------------------
+struct F2 {
+  unsigned long long v;
+};
+__device__ __forceinline__ F2 mk2(float lo, float hi) {
+  F2 r;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(r.v) : "f"(lo), "f"(hi));
+  return r;
+}
+__device__ __forceinline__ void get2(F2 p, float& lo, float& hi) {
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(lo), "=f"(hi) : "l"(p.v));
+}
+__device__ __forceinline__ F2 dup2(float x) { return mk2(x, x); }
+__device__ __forceinline__ F2 add2(F2 a, F2 b) {
+  F2 r;
+  asm("add.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 mul2(F2 a, F2 b) {
+  F2 r;
+  asm("mul.rn.ftz.f32x2 %0, %1, %2;" : "=l"(r.v) : "l"(a.v), "l"(b.v));
+  return r;
+}
+__device__ __forceinline__ F2 fma2(F2 a, F2 b, F2 c) {
+  F2 r;
+  asm("fma.rn.ftz.f32x2 %0, %1, %2, %3;" : "=l"(r.v) : "l"(a.v), "l"(b.v), "l"(c.v));
+  return r;
+}
+
 // r = |x| from r^2 (0 for coincident points)
 template <class R> __device__ __forceinline__ R radius(R r2) {
   return r2 > R(0) ? sqrt_(r2) : R(0);
