@@ -40,12 +40,16 @@ Layout make_layout(const crk_params& p, int64_t n, int32_t nb) {
   };
   L.hdr = take(sizeof(DevHeader));
   L.box_L = take(8 * (size_t)std::max(nb, 1));
+  L.box_scale = take(16 * (size_t)std::max(nb, 1));
   L.hbox = take(4 * (size_t)std::max(nb, 1));
   L.key0 = take(8 * N);
   L.key1 = take(8 * N);
   L.val0 = take(4 * N);
   L.val1 = take(4 * N);
-  L.hist = take(4 * 256 * (size_t)std::max<int64_t>(L.ntiles, 1));
+  // digit counts: one set of the long sort's tiles, or up to eight digits of the
+  // short sort's (at most 152 tiles, no more than the long sort's)
+  L.hist = take(4 * 256 * (size_t)std::max<int64_t>(
+                              {L.ntiles, 8 * std::min<int64_t>(L.ntiles, 152), 1}));
   int64_t scan_n = std::max<int64_t>({256 * L.ntiles, n + 1});
   L.scan_tmp = take(scan_tmp_bytes(scan_n));
   L.perm = take(4 * N);
@@ -54,12 +58,7 @@ Layout make_layout(const crk_params& p, int64_t n, int32_t nb) {
   L.hs = take(R * N);
   L.ms = take(R * N);
   L.us = take(R * N);
-  L.aabb = take(4 * 6 * NT);
-  L.hmaxn = take(4 * NT);
-  L.brange = take(4 * 2 * NT);
-  L.child = take(4 * 2 * NI);
-  L.parent = take(4 * NT);
-  L.visit = take(4 * NI);
+  L.bkey = take(8 * (size_t)L.nbk);
   L.p4 = take(16 * N);
   L.nrec = take(4 * kNodeRec * NT);
   L.cnt_g = take(4 * N);

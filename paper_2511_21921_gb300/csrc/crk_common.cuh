@@ -313,10 +313,10 @@ struct Layout {
   int64_t n = 0, nb = 0, nw = 0, nbk = 0, ni = 0, nt = 0, ntiles = 0, cap = 0, cap_pp = 0;
   int prec = 1;
   size_t total = 0;
-  size_t hdr = 0, box_L = 0, hbox = 0;
+  size_t hdr = 0, box_L = 0, box_scale = 0, hbox = 0;
   size_t key0 = 0, key1 = 0, val0 = 0, val1 = 0, hist = 0, scan_tmp = 0;
   size_t perm = 0, boxid = 0, xs = 0, hs = 0, ms = 0, us = 0, vs = 0;
-  size_t aabb = 0, hmaxn = 0, brange = 0, child = 0, parent = 0, visit = 0;
+  size_t bkey = 0;  // key of each bucket's first particle
   // the list build's packed copies: float4 (x, y, z, h) per sorted particle
   // and one 64-byte record per tree node (bounds, h_max, box range, children)
   size_t p4 = 0, nrec = 0;

@@ -40,10 +40,7 @@ template <class R> struct SubArgs {
   const int32_t* boxid;
   const int32_t* perm;
   const uint8_t* spec;  // nullptr: all gas; winds are skipped (they are subgrid particles)
-  const float* aabb;
-  const float* hmaxn;
-  const int32_t* brange;
-  const int32_t* child;
+  const float* nrec;    // node records: bounds, h_max, box range, children
   DevHeader* hdr;
   // volume
   R n_h;
@@ -112,12 +109,20 @@ __device__ bool walk(const SubArgs<R>& a, int32_t b, const double* p, double L, 
     __syncwarp();
     if (node >= 0 && !index_ok(a.hdr, node, a.nt)) node = -1;
     bool ov = false;
-    if (node >= 0 && b >= a.brange[node] && b <= a.brange[a.nt + node]) {
-      const float R_ = (reach_fixed >= 0.f ? reach_fixed : a.hmaxn[node]) * 1.00001f + 1e-6f * Lf;
+    float4 r0 = {}, r1 = {}, r2 = {};
+    if (node >= 0) {
+      const float4* rec = reinterpret_cast<const float4*>(a.nrec + (int64_t)node * kNodeRec);
+      r0 = __ldg(rec);
+      r1 = __ldg(rec + 1);
+      r2 = __ldg(rec + 2);
+    }
+    if (node >= 0 && b >= __float_as_int(r1.w) && b <= __float_as_int(r2.x)) {
+      const float R_ = (reach_fixed >= 0.f ? reach_fixed : r1.z) * 1.00001f + 1e-6f * Lf;
+      const float nlo[3] = {r0.x, r0.y, r0.z}, nhi[3] = {r0.w, r1.x, r1.y};
       float g2 = 0.f;
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
-        const float lo = a.aabb[c * a.nt + node], hi = a.aabb[(3 + c) * a.nt + node];
+        const float lo = nlo[c], hi = nhi[c];
         float dd = pf[c] - 0.5f * (lo + hi);
         if (dd > hLf) dd -= Lf;
         else if (dd < -hLf) dd += Lf;
@@ -131,8 +136,8 @@ __device__ bool walk(const SubArgs<R>& a, int32_t b, const double* p, double L, 
     if (sp + 2 * __popc(mi) > kSubStack) return false;
     if (ov && !leaf) {
       const int at = sp + 2 * __popc(mi & lt);
-      stk[at] = a.child[2 * node];
-      stk[at + 1] = a.child[2 * node + 1];
+      stk[at] = __float_as_int(r2.y);
+      stk[at + 1] = __float_as_int(r2.z);
     }
     sp += 2 * __popc(mi);
     __syncwarp();
@@ -246,10 +251,7 @@ static SubArgs<R> sub_args(Plan* P, char* ws, int64_t n_s, const int64_t* box_of
   a.boxid = reinterpret_cast<const int32_t*>(ws + Ly.boxid);
   a.perm = reinterpret_cast<const int32_t*>(ws + Ly.perm);
   a.spec = P->species ? reinterpret_cast<const uint8_t*>(ws + Ly.spec) : nullptr;
-  a.aabb = reinterpret_cast<const float*>(ws + Ly.aabb);
-  a.hmaxn = reinterpret_cast<const float*>(ws + Ly.hmaxn);
-  a.brange = reinterpret_cast<const int32_t*>(ws + Ly.brange);
-  a.child = reinterpret_cast<const int32_t*>(ws + Ly.child);
+  a.nrec = reinterpret_cast<const float*>(ws + Ly.nrec);
   a.hdr = reinterpret_cast<DevHeader*>(ws + Ly.hdr);
   return a;
 }

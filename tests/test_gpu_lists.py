@@ -47,3 +47,34 @@ def test_lists_match_the_double_predicate(precision, scale, n):
     for mode, want in (("gather", g), ("union", u)):
         got = _rows(s.neighbors_csr(mode))
         assert got == [np.nonzero(r)[0].tolist() for r in want]
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 2049, 155648, 155649, 311297, 622592, 622593])
+def test_pairs_at_the_sort_tile_edges(n):
+    """Sizes where the sort's tiles or its dispatch change, several boxes of two
+    sides: the number of pairs and the lists of sampled particles from a k-d tree."""
+    from scipy.spatial import cKDTree
+    rng = np.random.default_rng(n)
+    off = np.array([0, n // 3, n // 3, n], np.int64)  # the middle box is empty
+    side = np.array([1.0, 1.0, 2.5])
+    x, h = np.empty((3, n)), np.empty(n)
+    total = 0
+    rows = {}
+    for b in range(3):
+        a, e = off[b], off[b + 1]
+        if e == a:
+            continue
+        x[:, a:e] = rng.random((3, e - a)) * side[b]
+        hb = np.float32(1.2 * side[b] * (e - a) ** (-1 / 3) if e - a > 27 else 0.3 * side[b])
+        h[a:e] = hb
+        t = cKDTree(x[:, a:e].T, boxsize=side[b])
+        total += t.count_neighbors(t, float(hb)) - (e - a)
+        for i in rng.integers(0, e - a, 20):
+            rows[a + i] = sorted(a + k for k in t.query_ball_point(x[:, a + i], float(hb)) if k != i)
+    s = Solver(n, 3, "mixed")
+    s.cell_build(torch.tensor(x, device="cuda"), torch.tensor(h, dtype=torch.float32, device="cuda"),
+                 box_off=torch.tensor(off, device="cuda"), box_L=torch.tensor(side, device="cuda"))
+    assert s.stats()["gather_pairs"] == s.stats()["union_pairs"] == total
+    row, col = (t.cpu().numpy() for t in s.neighbors_csr("gather"))
+    for i, want in rows.items():
+        assert col[row[i]:row[i + 1]].tolist() == want
