@@ -122,8 +122,10 @@ class Solver:
             self.n, self.nb, self._wsp = n, nb, ws
             if not check:
                 return self
+            # the counters carry the status word; only an error is read (and
+            # cleared) a second time
             st = L.crk_stats_get(self.plan, _stream(), ws)
-            code = L.crk_status_poll(self.plan, _stream(), ws)
+            code = L.crk_status_poll(self.plan, _stream(), ws) if st.status else L.CRK_OK
             if code == L.CRK_ENOMEM and st.list_slots > st.list_capacity:
                 self._regrow(int(math.ceil(st.list_slots * 1.05)) + 8)
                 continue
@@ -283,7 +285,11 @@ class Solver:
         if box_off_s is not None:
             return box_off_s
         assert self.nb == 1, "pass box_off_s for a multi-box build"
-        return torch.tensor([0, n_s], dtype=torch.int64, device=self.device)
+        # made once per count: the copy from the host would wait for the stream
+        if getattr(self, "_sub_key", None) != n_s:
+            self._sub_default = torch.tensor([0, n_s], dtype=torch.int64, device=self.device)
+            self._sub_key = n_s
+        return self._sub_default
 
     def subgrid_volume(self, x_s, h_s, n_h=2.25, box_off_s=None, want_h=True):
         """Scatter volumes of subgrid particles (and n_h V^(1/3))."""
