@@ -315,14 +315,15 @@ template <class R, bool VAR = false> struct PassA2 {
       gix[p] = gvi[3 * p] * d[0] + gvi[3 * p + 1] * d[1] + gvi[3 * p + 2] * d[2];
       gjx[p] = gvj[3 * p] * d[0] + gvj[3 * p + 1] * d[1] + gvj[3 * p + 2] * d[2];
     }
-    R phi = R(0), phi0 = R(0), damp = R(1), z = R(0), pa = R(0), pb = R(0);
+    R phi = R(0), phi0 = R(0), damp = R(1), z = R(0), pa = R(0), pb = R(0), is = R(0);
     bool dampon = false;
     const R ihmin = fmin(ihi, ihj);
     const R eta = r * ihmin;
     if (a.av.limiter) {
       pa = d[0] * gix[0] + d[1] * gix[1] + d[2] * gix[2];
       pb = d[0] * gjx[0] + d[1] * gjx[1] + d[2] * gjx[2];
-      phi0 = PairC2<R>::limiter_phi(pa, pb);
+      is = recip(pa + pb);
+      phi0 = PairC2<R>::limiter_phi(pa, pb, is);
       phi = phi0;
       if (eta < a.av.eta_crit) {
         dampon = true;
@@ -341,7 +342,8 @@ template <class R, bool VAR = false> struct PassA2 {
     const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
     const R Di = r2 * (ihi * ihi) + a.av.eps2;
     const R Dj = r2 * (ihj * ihj) + a.av.eps2;
-    const R tmi = vx * ihi / Di, tmj = vx * ihj / Dj;
+    const R iDi = recip(Di), iDj = recip(Dj);
+    const R tmi = quot(vx * ihi, Di, iDi), tmj = quot(vx * ihj, Dj, iDj);
     const R mui = tmi < R(0) ? tmi : R(0);
     const R muj = tmj < R(0) ? tmj : R(0);
     const R qai = ri[RC::C2_QA], qbi = ri[RC::C2_QB], qaj = rj[RC::C2_QA], qbj = rj[RC::C2_QB];
@@ -429,13 +431,13 @@ template <class R, bool VAR = false> struct PassA2 {
     R vxb = R(0), r2b = R(0), ihib = R(0), rb = R(0);
     R db[3] = {R(0), R(0), R(0)};
     if (tmi < R(0)) {
-      vxb += muib * ihi / Di;
-      ihib += muib * (vx / Di) * (R(1) - R(2) * r2 * (ihi * ihi) / Di);
-      r2b += muib * (-vx * (ihi * ihi * ihi) / (Di * Di));
+      vxb += quot(muib * ihi, Di, iDi);
+      ihib += muib * quot(vx, Di, iDi) * (R(1) - quot(R(2) * r2 * (ihi * ihi), Di, iDi));
+      r2b += muib * quot(-vx * (ihi * ihi * ihi), Di * Di, iDi * iDi);
     }
     if (tmj < R(0)) {
-      vxb += mujb * ihj / Dj;
-      r2b += mujb * (-vx * (ihj * ihj * ihj) / (Dj * Dj));
+      vxb += quot(mujb * ihj, Dj, iDj);
+      r2b += mujb * quot(-vx * (ihj * ihj * ihj), Dj * Dj, iDj * iDj);
     }
     R vhb[3], gsum[3];
 #pragma unroll
@@ -462,9 +464,9 @@ template <class R, bool VAR = false> struct PassA2 {
       }
       if (pa * pb > R(0)) {
         const R sm = pa + pb;
-        const R s3 = sm * sm * sm;
-        const R pab = phi0b * R(4) * pb * (pb - pa) / s3;
-        const R pbb = phi0b * R(4) * pa * (pa - pb) / s3;
+        const R s3 = sm * sm * sm, is3 = is * is * is;
+        const R pab = quot(phi0b * R(4) * pb * (pb - pa), s3, is3);
+        const R pbb = quot(phi0b * R(4) * pa * (pa - pb), s3, is3);
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
           db[p] += pab * gix[p] + pbb * gjx[p];

@@ -591,11 +591,11 @@ __device__ __forceinline__ R energy_share(bool split, R E, R ui, R uj) {
 template <class R> struct PairC2 {
   using RC = Rec<R>;
   // limiter phi from a = x.gv_i.x, b = x.gv_j.x:  4ab/(a+b)^2 when ab > 0
-  __device__ static __forceinline__ R limiter_phi(R a, R b) {
+  __device__ static __forceinline__ R limiter_phi(R a, R b, R is) {  // is: recip(a + b)
     const R ab = a * b;
     if (!(ab > R(0))) return R(0);
     const R sm = a + b;
-    return R(4) * ab / (sm * sm);
+    return quot(R(4) * ab, sm * sm, is * is);
   }
   template <bool VAR = false>
   __device__ static __forceinline__ void force(const R* ri, const R* rj, const R* d, R r2,
@@ -623,7 +623,7 @@ template <class R> struct PairC2 {
     if (av.limiter) {
       const R pa = d[0] * gix[0] + d[1] * gix[1] + d[2] * gix[2];
       const R pb = d[0] * gjx[0] + d[1] * gjx[1] + d[2] * gjx[2];
-      phi = limiter_phi(pa, pb);
+      phi = limiter_phi(pa, pb, recip(pa + pb));
       const R eta = r * fmin(ihi, ihj);
       if (eta < av.eta_crit) {
         const R z = (eta - av.eta_crit) / av.eta_fold;
@@ -636,8 +636,9 @@ template <class R> struct PairC2 {
     for (int p = 0; p < 3; ++p)
       vh[p] = (ri[RC::C2_VEL + p] - rj[RC::C2_VEL + p]) - hphi * (gix[p] + gjx[p]);
     const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
-    R mui = vx * ihi / (r2 * (ihi * ihi) + av.eps2);
-    R muj = vx * ihj / (r2 * (ihj * ihj) + av.eps2);
+    const R Di = r2 * (ihi * ihi) + av.eps2, Dj = r2 * (ihj * ihj) + av.eps2;
+    R mui = quot(vx * ihi, Di, recip(Di));
+    R muj = quot(vx * ihj, Dj, recip(Dj));
     mui = mui < R(0) ? mui : R(0);
     muj = muj < R(0) ? muj : R(0);
     const R Qi = mui * (ri[RC::C2_QB] * mui - ri[RC::C2_QA]);
