@@ -595,7 +595,7 @@ template <class R> struct PairC2 {
     const R ab = a * b;
     if (!(ab > R(0))) return R(0);
     const R sm = a + b;
-    return quot(R(4) * ab, sm * sm, is * is);
+    return quot_pow(R(4) * ab, sm * sm, is * is, sm);
   }
   template <bool VAR = false>
   __device__ static __forceinline__ void force(const R* ri, const R* rj, const R* d, R r2,
@@ -626,7 +626,7 @@ template <class R> struct PairC2 {
       phi = limiter_phi(pa, pb, recip(pa + pb));
       const R eta = r * fmin(ihi, ihj);
       if (eta < av.eta_crit) {
-        const R z = (eta - av.eta_crit) / av.eta_fold;
+        const R z = quot(eta - av.eta_crit, recip(av.eta_fold));
         phi = phi * exp_(-(z * z));
       }
     }
@@ -637,8 +637,8 @@ template <class R> struct PairC2 {
       vh[p] = (ri[RC::C2_VEL + p] - rj[RC::C2_VEL + p]) - hphi * (gix[p] + gjx[p]);
     const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
     const R Di = r2 * (ihi * ihi) + av.eps2, Dj = r2 * (ihj * ihj) + av.eps2;
-    R mui = quot(vx * ihi, Di, recip(Di));
-    R muj = quot(vx * ihj, Dj, recip(Dj));
+    R mui = quot(vx * ihi, recip(Di));
+    R muj = quot(vx * ihj, recip(Dj));
     mui = mui < R(0) ? mui : R(0);
     muj = muj < R(0) ? muj : R(0);
     const R Qi = mui * (ri[RC::C2_QB] * mui - ri[RC::C2_QA]);
