@@ -612,7 +612,7 @@ __global__ void k_lbvh(const uint64_t* __restrict__ bkey, const int32_t* __restr
 }
 
 // ---------------------------------------------------------------------------
-// neighbor lists: one thread per sorted particle traverses the tree
+// neighbor lists: one warp per 32 sorted particles traverses the tree
 // ---------------------------------------------------------------------------
 // r^2 as the definition forms it (no contraction)
 __device__ __forceinline__ double norm2(const double* d) {
@@ -649,7 +649,7 @@ __device__ __forceinline__ double exact_r2(const double* __restrict__ xd, int64_
 // whole group (separately for each box present in the group): nodes are
 // tested 32 at a time against the group's bounding box grown by
 // max(h over the group, h_max of the node); overlapping buckets are staged
-// 4 at a time (32 particles) in shared memory and every lane tests its own
+// 4 or 8 at a time (32 or 64 particles) in shared memory and every lane tests its own
 // particle against all 32.  Traversal order is
 // fixed, so the counting and the filling pass see the same entries.
 // Center, half extent and largest h of the lanes with `in` set (all lanes
@@ -679,42 +679,47 @@ __device__ __forceinline__ void group_bounds(bool in, const float* p, float h, f
   }
 }
 
-constexpr int kNbrWarps = 4;
-// Resident blocks per SM (80 registers a thread, 16 KB of shared memory a block).
-// The build is bound by issue (60 % active): a third of its time is the tree
-// walk and the staging of candidates, a fifth the 32-candidate tests, a quarter
-// the emission of hits.  262,144 / 2.1 M / 16.8 M particles: 0.685 / 4.5 / 33.8 ms
-// with distances and bands evaluated again per hit, 0.558 / 3.68 / 27.0 ms with
-// the masks; 5 blocks 0.572 / 3.97 / 29.5, 8 blocks (64 registers) 0.590 / 3.66 /
-// 26.4.
-constexpr int kNbrBlocks = 6;
+// Resident blocks per SM, of one warp each (80 registers a thread, 5 KB of shared
+// memory a block).  The walks of neighboring groups differ by a factor of two and
+// more in length, so a block of four warps held its place until the slowest of them
+// ended.  The build is bound by issue: of a warp's time a quarter each is the tree
+// walk, the staging of candidates and the emission of hits, a sixth the
+// 32-candidate tests.  Lists of 30,011 / 262,144 / 2.1 M particles: 0.215 / 0.685 /
+// 4.5 ms with distances and bands evaluated again per hit, 0.201 / 0.556 / 3.63 with
+// the masks, 0.186 / 0.537 / 3.58 with eight buckets staged at once and box numbers
+// read only where a bucket holds two boxes, 0.164 / 0.470 / 3.08 with blocks of one
+// warp (20 a SM 0.174 / 0.519 / 3.52, 28 a SM 0.178 / 0.476 / 3.05; two warps a block
+// 0.188 / 0.535 / 3.48).
+constexpr int kNbrBlocks = 24;
 // Node stack of a warp.  Taking 32 nodes a step adds at most 32 to it; from
 // three quarters on the walk takes one node a step, which adds at most one per
 // level of the tree (94 at most: 64 key bits and 30 index bits), so it cannot
 // overflow.  (The deepest seen with 32 a step: 268, the clumpy 128^3 box.)
 constexpr int kNodeStack = 512;
+// Staged candidates: a ring of three stages of 32, since up to 64 are appended to
+// at most 31 that wait.
+constexpr int kStage = 96;
 
 template <class R>
-__global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
+__global__ void __launch_bounds__(32, kNbrBlocks) k_nbr(
     const uint64_t* __restrict__ keys, const R* __restrict__ hs, const int32_t* __restrict__ boxid,
     const double* __restrict__ box_L, int64_t n, int64_t nbk, int64_t ni, int64_t nt,
     const float* __restrict__ nrec, const float4* __restrict__ p4, int32_t* __restrict__ cnt_g, int32_t* __restrict__ cnt_s, int32_t* __restrict__ wlen_g,
     int32_t* __restrict__ wlen_s, uint32_t* __restrict__ ell, int64_t cap_pp, DevHeader* hdr,
     const double* __restrict__ xd, const int32_t* __restrict__ perm,
     const float* __restrict__ hbox) {
-  __shared__ int32_t stk[kNbrWarps][kNodeStack];
-  __shared__ int32_t cand[kNbrWarps][64];
+  __shared__ int32_t stk[kNodeStack];
+  // candidate buckets; the top bit marks one that may hold particles of two boxes
+  __shared__ int32_t cand[64];
   // staged candidates, one array per component so that four (a 128-bit load)
   // arrive at once: float position (of the nearest image, where one serves the
   // whole group), h^2, its rounding band, index; and the slot of each lane's own
-  // particle (-1: not staged)
-  __shared__ float4 stage[kNbrWarps][5][16];
-  __shared__ int32_t sj[kNbrWarps][64];
-  __shared__ int32_t self_at[kNbrWarps][32];
-  const int wib = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int64_t w = (int64_t)blockIdx.x * kNbrWarps + wib;
-  const int64_t nw = (n + 31) / 32;
-  if (w >= nw) return;  // whole warp
+  // particle (-kStage: not staged)
+  __shared__ float4 stage[5][kStage / 4];
+  __shared__ int32_t sj[kStage];
+  __shared__ int32_t self_at[32];
+  const int lane = threadIdx.x;
+  const int64_t w = blockIdx.x;
   const uint32_t lt = (1u << lane) - 1u;
   const int64_t s = w * 32 + lane;
   const bool live = s < n;
@@ -789,15 +794,16 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
       }
     }
     int sp = 0, nc = 0;
-    int ns = 0;  // candidates waiting in the stage
+    int base = 0;  // first slot of the stage that is tested next
+    int ns = 0;    // candidates waiting from there on
     const float hi2f = hi * hi;
     const float tol_i = list_band(hi, Lf);
     const float iLf = 1.f / Lf;
     // outside this range of box sides float squares could leave the float range:
     // every pair is then decided exactly
     const bool in_range = Lf > 1e-6f && Lf < 1e15f;
-    float* sx = reinterpret_cast<float*>(stage[wib]);  // component c, slot k: sx[64 c + k]
-    self_at[wib][lane] = -1;
+    float* sx = reinterpret_cast<float*>(stage);  // component c, slot k: sx[kStage c + k]
+    self_at[lane] = -kStage;
     // Tests the first 32 staged candidates (`filled` of them valid) against the
     // lane's particle and appends the hits to its column.  Branch-free into
     // three bit masks, two candidates per packed operation: gather
@@ -815,6 +821,7 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
       const D2 minus = dup2(-1.f), nhi2 = dup2(-hi2f);
       const D2 iL2 = dup2(iLf), nL2 = dup2(-Lf), mg = dup2(12582912.f), nmg = dup2(-12582912.f);
       uint32_t G = 0u, S = 0u, X = 0u;
+      const int b4 = base >> 2;
       auto image = [&](D2 d) {
         if constexpr (decltype(wrap)::value)
           d = fma2(add2(fma2(d, iL2, mg), nmg), nL2, d);
@@ -822,8 +829,8 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
       };
 #pragma unroll
       for (int q = 7; q >= 0; --q) {
-        const float4 tx = stage[wib][0][q], ty = stage[wib][1][q], tz = stage[wib][2][q];
-        const float4 th = stage[wib][3][q], tt = stage[wib][4][q];
+        const float4 tx = stage[0][b4 + q], ty = stage[1][b4 + q], tz = stage[2][b4 + q];
+        const float4 th = stage[3][b4 + q], tt = stage[4][b4 + q];
         const float* vx = &tx.x;
         const float* vy = &ty.x;
         const float* vz = &tz.x;
@@ -848,14 +855,16 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
         }
       }
       uint32_t valid = filled < 32 ? (1u << filled) - 1u : kFull;
-      const int own = self_at[wib][lane];
-      self_at[wib][lane] = own >= 32 ? own - 32 : -1;
-      if (own >= 0 && own < 32) valid &= ~(1u << own);
+      const unsigned own = (unsigned)(self_at[lane] - base);
+      if (own < 32u) {
+        valid &= ~(1u << own);
+        self_at[lane] = -kStage;
+      }
       X = in_range ? X & valid : valid;
       while (X) {
         const int k = __ffs(X) - 1;
         X &= X - 1u;
-        const int32_t j = sj[wib][k];
+        const int32_t j = sj[base + k];
         const double r2d = exact_r2(xd, n, perm[s], perm[j], Ld);
         const uint32_t bit = 1u << k;
         G = r2d < sq((double)hs[s]) ? G | bit : G & ~bit;
@@ -868,7 +877,7 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
         const int k = __ffs(U) - 1;
         U &= U - 1u;
         const uint32_t g = (G >> k) & 1u;
-        const uint32_t e = (uint32_t)sj[wib][k] | g << 31 | ((S >> k) & 1u) << 30;
+        const uint32_t e = (uint32_t)sj[base + k] | g << 31 | ((S >> k) & 1u) << 30;
         const int at = g ? kg : (int)cap_pp - 1 - ks;
         if (kg + ks < (int)cap_pp) col[at * 32] = e;
         kg += (int)g;
@@ -881,18 +890,18 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
         else test_stage(filled, std::true_type{});
       }
     };
-    if (lane == 0) stk[wib][0] = (ni > 0) ? 0 : (int32_t)ni;
+    if (lane == 0) stk[0] = (ni > 0) ? 0 : (int32_t)ni;
     sp = 1;
     __syncwarp();
     while (sp > 0 || nc > 0) {
       if (sp > 0) {
         // one node at a time (depth first) once the stack is three quarters full
         const int take = sp > kNodeStack * 3 / 4 ? 1 : (sp < 32 ? sp : 32);
-        const int32_t node = lane < take ? stk[wib][sp - take + lane] : -1;
+        const int32_t node = lane < take ? stk[sp - take + lane] : -1;
         sp -= take;
         cnt_nodes += take;
         __syncwarp();
-        bool ov = false;
+        bool ov = false, one_box = false;
         int2 ch = make_int2(0, 0);
         if (node >= 0) {
           // the whole node record (bounds, h_max, box range, children) in
@@ -905,8 +914,11 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
           const float* lo = nr;
           const float* hi_ = nr + 3;
           ch = make_int2(__float_as_int(nr[9]), __float_as_int(nr[10]));
+          one_box = b0 == b1;
           if (b >= b0 && b <= b1) {
-            const float R_ = fmaxf(hg, hm) * 1.00001f + 1e-6f * Lf;
+            // rounded as written (fma_, rmul): which nodes overlap sets the order of
+            // the lists, and with it the sums' rounding
+            const float R_ = fma_(1e-6f, Lf, rmul(fmaxf(hg, hm), 1.00001f));
             float g2 = 0.f;
 #pragma unroll
             for (int a = 0; a < 3; ++a) {
@@ -914,7 +926,7 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
               if (dd > halfLf) dd -= Lf;
               else if (dd < -halfLf) dd += Lf;
               dd = fabsf(dd) - ge[a] - 0.5f * (hi_[a] - lo[a]);
-              if (dd > 0.f) g2 += dd * dd;
+              if (dd > 0.f) g2 = fma_(dd, dd, g2);
             }
             ov = g2 <= R_ * R_;
           }
@@ -922,7 +934,8 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
         const bool leaf = node >= ni;
         const unsigned ml = __ballot_sync(kFull, ov && leaf);
         const unsigned mi = __ballot_sync(kFull, ov && !leaf);
-        if (ov && leaf) cand[wib][nc + __popc(ml & lt)] = node - (int32_t)ni;
+        if (ov && leaf)
+          cand[nc + __popc(ml & lt)] = (node - (int32_t)ni) | (one_box ? 0 : (int32_t)0x80000000);
         nc += __popc(ml);
         const int npush = 2 * __popc(mi);
         if (sp + npush > kNodeStack) {
@@ -931,74 +944,75 @@ __global__ void __launch_bounds__(kNbrWarps * 32, kNbrBlocks) k_nbr(
         }
         if (ov && !leaf) {
           const int at = sp + 2 * __popc(mi & lt);
-          stk[wib][at] = ch.x;
-          stk[wib][at + 1] = ch.y;
+          stk[at] = ch.x;
+          stk[at + 1] = ch.y;
         }
         sp += npush;
         __syncwarp();
       }
       while (nc >= 4 || (sp == 0 && nc > 0)) {
+        // stage the particles of the last four candidate buckets, or of the last
+        // two fours: the loads of both are in flight together
         const int take = nc < 4 ? nc : 4;
-        nc -= take;
-        cnt_buckets += take;
-        // stage the particles of buckets cand[nc .. nc+take)
+        const bool two = nc >= 8;
+        cnt_buckets += two ? 8 : take;
         const int kb = lane >> 3;
+        int64_t jj[2];
+        float4 pj[2];
+        int32_t bj[2];
+#pragma unroll
+        for (int t = 0; t < 2; ++t) {
+          const bool has = t == 0 ? kb < take : two;
+          const int32_t c = has ? cand[(t == 0 ? nc - take : nc - 8) + kb] : 0;
+          jj[t] = (int64_t)(c & 0x7fffffff) * kBucket + (lane & 7);
+          pj[t] = make_float4(0.f, 0.f, 0.f, 0.f);
+          bj[t] = -1;
+          if (has && jj[t] < n) {
+            pj[t] = __ldg(p4 + jj[t]);
+            bj[t] = c < 0 ? __ldg(boxid + jj[t]) : b;
+          }
+        }
+        nc -= two ? 8 : take;
         // A particle that lies farther from the group's box than
         // max(h_group, h_j) cannot be a union neighbor of any lane and is
         // dropped here; the others are appended to the stage, which is tested
         // once it holds 32.  Dropping preserves the order of the survivors, so
         // every list comes out exactly as without the filter.
-        int64_t j = -1;
-        float q[3] = {0.f, 0.f, 0.f}, hj = 0.f;
-        bool pass = false;
-        if (kb < take) {
-          const int64_t jj = (int64_t)cand[wib][nc + kb] * kBucket + (lane & 7);
-          if (jj < n) {
-            const int32_t bj = __ldg(boxid + jj);
-            const float4 pj = __ldg(p4 + jj);
-            q[0] = pj.x;
-            q[1] = pj.y;
-            q[2] = pj.z;
-            hj = pj.w;
-            if (bj == b) {
-              j = jj;
-              float g2 = 0.f;
 #pragma unroll
-              for (int a = 0; a < 3; ++a) {
-                const float dd = gc[a] - q[a];
-                const float qn = q[a] + (dd > halfLf ? Lf : (dd < -halfLf ? -Lf : 0.f));
-                const float o = fabsf(qn - gc[a]) - ge[a];
-                if (o > 0.f) g2 += o * o;
-                if (one_image) q[a] = qn;
-              }
-              const float Rj = fmaxf(hg, hj) * 1.00001f + 1e-6f * Lf;
-              pass = g2 <= Rj * Rj;
-            }
+        for (int t = 0; t < 2; ++t) {
+          float q[3] = {pj[t].x, pj[t].y, pj[t].z};
+          const float hj = pj[t].w;
+          float g2 = 0.f;
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            const float dd = gc[a] - q[a];
+            const float qn = q[a] + (dd > halfLf ? Lf : (dd < -halfLf ? -Lf : 0.f));
+            const float o = fabsf(qn - gc[a]) - ge[a];
+            if (o > 0.f) g2 += o * o;
+            if (one_image) q[a] = qn;
           }
-        }
-        const unsigned mp = __ballot_sync(kFull, pass);
-        if (pass) {
-          const int at = ns + __popc(mp & lt);
+          const float Rj = fmaxf(hg, hj) * 1.00001f + 1e-6f * Lf;
+          const bool pass = bj[t] == b && g2 <= Rj * Rj;
+          const unsigned mp = __ballot_sync(kFull, pass);
+          if (pass) {
+            int at = base + ns + __popc(mp & lt);
+            at -= at >= kStage ? kStage : 0;
 #pragma unroll
-          for (int a = 0; a < 3; ++a) sx[64 * a + at] = q[a];
-          sx[192 + at] = hj * hj;
-          sx[256 + at] = list_band(hj, Lf);
-          sj[wib][at] = (int32_t)j;
-          if ((j >> 5) == w) self_at[wib][j & 31] = at;
+            for (int a = 0; a < 3; ++a) sx[kStage * a + at] = q[a];
+            sx[kStage * 3 + at] = hj * hj;
+            sx[kStage * 4 + at] = list_band(hj, Lf);
+            sj[at] = (int32_t)jj[t];
+            if ((jj[t] >> 5) == w) self_at[jj[t] & 31] = at;
+          }
+          ns += __popc(mp);
         }
-        ns += __popc(mp);
         __syncwarp();
-        if (ns >= 32) {
+        while (ns >= 32) {
           flush(32);
-          __syncwarp();
-          if (lane < ns - 32) {
-#pragma unroll
-            for (int a = 0; a < 5; ++a) sx[64 * a + lane] = sx[64 * a + 32 + lane];
-            sj[wib][lane] = sj[wib][32 + lane];
-          }
+          base = base == kStage - 32 ? 0 : base + 32;
           ns -= 32;
-          __syncwarp();
         }
+        __syncwarp();
       }
     }
     if (ns > 0) {
@@ -1316,10 +1330,9 @@ crk_status cell_build_impl(Plan* plan, cudaStream_t st, char* ws, int64_t n, int
   int32_t* wlen_g = reinterpret_cast<int32_t*>(ws + Ly.wlen_g);
   int32_t* wlen_s = reinterpret_cast<int32_t*>(ws + Ly.wlen_s);
   uint32_t* ell = reinterpret_cast<uint32_t*>(ws + Ly.ell);
-  const unsigned gw = (unsigned)((Ly.nw + kNbrWarps - 1) / kNbrWarps);
-  k_nbr<R><<<gw, kNbrWarps * 32, 0, st>>>(k0, hs, boxid, wbox, n, nbk, ni, nt, nrec, p4,
-                                          cnt_g, cnt_s, wlen_g, wlen_s, ell, Ly.cap_pp, hdr, x,
-                                          perm, reinterpret_cast<const float*>(hbox));
+  k_nbr<R><<<(unsigned)Ly.nw, 32, 0, st>>>(k0, hs, boxid, wbox, n, nbk, ni, nt, nrec, p4, cnt_g,
+                                             cnt_s, wlen_g, wlen_s, ell, Ly.cap_pp, hdr, x, perm,
+                                             reinterpret_cast<const float*>(hbox));
   int32_t* cost = reinterpret_cast<int32_t*>(ws + Ly.item_cost);
   int32_t* seq_cost = reinterpret_cast<int32_t*>(ws + Ly.seq_cost);
   k_balance<<<(unsigned)((n + kBalance - 1) / kBalance), kBalance, 0, st>>>(
