@@ -285,11 +285,10 @@ class Solver:
         if box_off_s is not None:
             return box_off_s
         assert self.nb == 1, "pass box_off_s for a multi-box build"
-        # made once per count: the copy from the host would wait for the stream
-        if getattr(self, "_sub_key", None) != n_s:
-            self._sub_default = torch.tensor([0, n_s], dtype=torch.int64, device=self.device)
-            self._sub_key = n_s
-        return self._sub_default
+        # [0, n_s] by a kernel: a copy from the host would wait for the stream
+        if n_s == 0:
+            return torch.zeros(2, dtype=torch.int64, device=self.device)
+        return torch.arange(0, n_s + 1, n_s, dtype=torch.int64, device=self.device)
 
     def subgrid_volume(self, x_s, h_s, n_h=2.25, box_off_s=None, want_h=True):
         """Scatter volumes of subgrid particles (and n_h V^(1/3))."""
