@@ -383,7 +383,8 @@ crk_status crk_cool_exact(crk_plan* plan, crk_stream_t stream, int64_t n,
  * workspace holds the state of a complete crk_moments + crk_rates call.
  * choice_out (optional, host int32[8]) receives the chosen variant per sweep,
  * ms_out (optional, host float[8][CRK_TUNE_VARIANTS]) the mean milliseconds of
- * every variant.  Synchronises.  Requires a built workspace. */
+ * every variant.  Synchronises.  Requires a built workspace.  A plan that was
+ * neither tuned nor given choices takes a variant by sweep, precision and size. */
 #define CRK_TUNE_VARIANTS 18
 crk_status crk_autotune(crk_plan* plan, crk_stream_t stream, void* ws, const void* m,
                         const void* v, const void* u, const void* g_dvdt, const void* g_dudt,

@@ -13,7 +13,8 @@
 // One warp per subgrid particle walks the gas bucket tree of the workspace
 // (the same tree the gas lists come from), 32 nodes at a time: for the scatter
 // volume a node is opened when the query point lies within the node's largest
-// gas h, for the deposit when the node lies within h_s.  Separations are formed in
+// gas h, for the deposit when the node lies within h_s.  The walk lists the buckets
+// in reach, which are then visited with a lane per gas particle.  Separations are formed in
 // the plan's precision from the double positions (double-float pairs in the
 // mixed form, exact in the FP64 form); kernel values likewise.
 // Deposits land in the caller's gas arrays with atomic adds (several subgrid
