@@ -91,8 +91,7 @@ Layout make_layout(const crk_params& p, int64_t n, int32_t nb) {
   L.flg = take(N);
   L.spec = take(N);
   L.Vgws = take(R * N);
-  L.act_pred = take(2 * 4 * N);
-  L.act_pos = take(2 * 4 * N);
+  L.act_part = take(8 * (N / Layout::kActTile + 1));
   L.items_r = take(4 * N);
   L.items_a = take(4 * N);
   L.items_bu = take(4 * N);

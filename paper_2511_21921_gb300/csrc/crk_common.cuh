@@ -357,8 +357,9 @@ struct Layout {
   size_t cnt_g = 0, cnt_s = 0, wlen_g = 0, wlen_s = 0, ell = 0;
   size_t rec_b1 = 0, rec_b2 = 0, rec_c1 = 0, rec_c2 = 0, coef = 0, Vs = 0, rhos = 0;
   size_t gvs = 0, Ds = 0;
-  // active-set evaluation: sorted flags, scan scratch, compacted work lists
-  size_t flg = 0, act_pred = 0, act_pos = 0, items_r = 0, items_a = 0;
+  // active-set evaluation: sorted flags, counts per tile, compacted work lists
+  static constexpr int kActTile = 2048;  // particles per count of the active-set lists
+  size_t flg = 0, act_part = 0, items_r = 0, items_a = 0;
   // length-balanced work list of the full union sweeps, the cost of each of
   // its 32-particle items and the items' longest-first order
   size_t items_bu = 0, item_cost = 0, item_order = 0;

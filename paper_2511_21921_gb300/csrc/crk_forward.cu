@@ -573,22 +573,100 @@ template crk_status forward_state_impl<double>(Plan*, cudaStream_t, char*, const
 // sweeps run over compacted lists of sorted indices; the records of the other
 // particles are packed from the caller's stored state.
 // ===========================================================================
-__global__ void k_active_flags(const uint8_t* __restrict__ flags, const int32_t* __restrict__ perm,
-                               int64_t n, uint8_t* __restrict__ flg, uint32_t* __restrict__ pr,
-                               uint32_t* __restrict__ pa) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s >= n) return;
-  const uint8_t f = flags[perm[s]];
-  const bool a = (f & 1) != 0, r = (f & 3) != 0;
-  flg[s] = (uint8_t)((a ? 1 : 0) | (r ? 2 : 0));
-  pr[s] = r ? 1u : 0u;
-  pa[s] = a ? 1u : 0u;
+// Two launches: flags in sorted order with their counts per tile of kActTile
+// particles, then every block adds the counts of the tiles before its own and
+// writes its tile's indices in order.  (Two scans of n flags and two compactions,
+// nine launches, took 0.044 ms of an active-set step of 262,144 particles; these
+// take 0.012.)
+constexpr int kActPer = 8, kActThreads = 256, kActTile = Layout::kActTile;
+static_assert(kActTile == kActPer * kActThreads, "a tile is one block's particles");
+
+__global__ void __launch_bounds__(kActThreads)
+    k_active_flags(const uint8_t* __restrict__ flags, const int32_t* __restrict__ perm, int64_t n,
+                   uint8_t* __restrict__ flg, uint2* __restrict__ part) {
+  __shared__ uint32_t sums[kActThreads / 32];
+  const int64_t base = (int64_t)blockIdx.x * kActTile + threadIdx.x;
+  uint32_t cnt = 0u;  // recompute set | active set << 16
+#pragma unroll
+  for (int q = 0; q < kActPer; ++q) {
+    const int64_t s = base + q * kActThreads;
+    if (s < n) {
+      const uint8_t f = flags[perm[s]];
+      const uint32_t a = (f & 1) ? 1u : 0u, r = (f & 3) ? 1u : 0u;
+      flg[s] = (uint8_t)(a | r << 1);
+      cnt += r | a << 16;
+    }
+  }
+  cnt = __reduce_add_sync(kFull, cnt);
+  if ((threadIdx.x & 31) == 0) sums[threadIdx.x >> 5] = cnt;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    uint32_t t = 0u;
+#pragma unroll
+    for (int w = 0; w < kActThreads / 32; ++w) t += sums[w];
+    part[blockIdx.x] = make_uint2(t & 0xffffu, t >> 16);
+  }
 }
 
-__global__ void k_compact(const uint32_t* __restrict__ pred, const uint32_t* __restrict__ pos,
-                          int64_t n, int32_t* __restrict__ items) {
-  const int64_t s = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (s < n && pred[s]) items[pos[s]] = (int32_t)s;
+__global__ void __launch_bounds__(kActThreads)
+    k_active_items(const uint8_t* __restrict__ flg, int64_t n, const uint2* __restrict__ part,
+                   int32_t* __restrict__ items_r, int32_t* __restrict__ items_a,
+                   int32_t* __restrict__ n_items) {
+  constexpr int kWarps = kActThreads / 32;
+  __shared__ uint32_t cnt[kActPer * kWarps];  // per 32 particles, then those before them
+  __shared__ uint2 before[kWarps];
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t base = (int64_t)blockIdx.x * kActTile + threadIdx.x;
+  uint2 mine = make_uint2(0u, 0u);
+  for (unsigned k = threadIdx.x; k < blockIdx.x; k += kActThreads) {
+    const uint2 v = part[k];
+    mine.x += v.x;
+    mine.y += v.y;
+  }
+  mine.x = __reduce_add_sync(kFull, mine.x);
+  mine.y = __reduce_add_sync(kFull, mine.y);
+  if (lane == 0) before[wid] = mine;
+  unsigned r[kActPer], a[kActPer];
+#pragma unroll
+  for (int q = 0; q < kActPer; ++q) {
+    const int64_t s = base + q * kActThreads;
+    const uint8_t f = s < n ? flg[s] : (uint8_t)0;
+    r[q] = __ballot_sync(kFull, (f & 2) != 0);
+    a[q] = __ballot_sync(kFull, (f & 1) != 0);
+    if (lane == 0) cnt[q * kWarps + wid] = __popc(r[q]) | __popc(a[q]) << 16;
+  }
+  __syncthreads();
+  if (wid == 0) {
+    const uint32_t c0 = cnt[2 * lane], c1 = cnt[2 * lane + 1];
+    uint32_t inc = c0 + c1;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t t = __shfl_up_sync(kFull, inc, o);
+      if (lane >= o) inc += t;
+    }
+    cnt[2 * lane] = inc - c0 - c1;
+    cnt[2 * lane + 1] = inc - c1;
+  }
+  __syncthreads();
+  uint32_t br = 0u, ba = 0u;
+#pragma unroll
+  for (int w = 0; w < kWarps; ++w) {
+    br += before[w].x;
+    ba += before[w].y;
+  }
+  const unsigned lt = (1u << lane) - 1u;
+#pragma unroll
+  for (int q = 0; q < kActPer; ++q) {
+    const uint32_t c = cnt[q * kWarps + wid];
+    const int32_t s = (int32_t)(base + q * kActThreads);
+    if ((r[q] >> lane) & 1u) items_r[br + (c & 0xffffu) + __popc(r[q] & lt)] = s;
+    if ((a[q] >> lane) & 1u) items_a[ba + (c >> 16) + __popc(a[q] & lt)] = s;
+  }
+  if (blockIdx.x + 1 == gridDim.x && threadIdx.x == 0) {
+    const uint2 own = part[blockIdx.x];
+    n_items[0] = (int32_t)(br + own.x);
+    n_items[1] = (int32_t)(ba + own.y);
+  }
 }
 
 // volume and coefficients of the particles that keep them
@@ -669,21 +747,16 @@ crk_status moments_active_impl(Plan* plan, cudaStream_t st, char* ws, const R* m
   cudaMemsetAsync(&c.hdr->queue[Q_B1], 0, 2 * sizeof(int32_t), st);
   if (n == 0) return CRK_OK;
   uint8_t* flg = reinterpret_cast<uint8_t*>(ws + Ly.flg);
-  uint32_t* pr = reinterpret_cast<uint32_t*>(ws + Ly.act_pred);
-  uint32_t* pa = pr + n;
-  uint32_t* qr = reinterpret_cast<uint32_t*>(ws + Ly.act_pos);
-  uint32_t* qa = qr + n;
+  uint2* part = reinterpret_cast<uint2*>(ws + Ly.act_part);
   int32_t* items_r = reinterpret_cast<int32_t*>(ws + Ly.items_r);
   int32_t* items_a = reinterpret_cast<int32_t*>(ws + Ly.items_a);
   const unsigned g = (unsigned)((n + 255) / 256);
   {
-    Phase ph(plan, st, "active_lists", 3 + 2 * scan_launches(n));
-    k_active_flags<<<g, 256, 0, st>>>(flags, c.perm, n, flg, pr, pa);
-    uint32_t* counts = reinterpret_cast<uint32_t*>(c.hdr->n_items);
-    exclusive_scan<uint32_t>(pr, qr, n, ws + Ly.scan_tmp, counts, st);
-    exclusive_scan<uint32_t>(pa, qa, n, ws + Ly.scan_tmp, counts + 1, st);
-    k_compact<<<g, 256, 0, st>>>(pr, qr, n, items_r);
-    k_compact<<<g, 256, 0, st>>>(pa, qa, n, items_a);
+    Phase ph(plan, st, "active_lists", 2);
+    const unsigned tiles = (unsigned)((n + kActTile - 1) / kActTile);
+    k_active_flags<<<tiles, kActThreads, 0, st>>>(flags, c.perm, n, flg, part);
+    k_active_items<<<tiles, kActThreads, 0, st>>>(flg, n, part, items_r, items_a,
+                                                  c.hdr->n_items);
   }
   R* rec_b1 = reinterpret_cast<R*>(ws + Ly.rec_b1);
   R* rec_b2 = reinterpret_cast<R*>(ws + Ly.rec_b2);
