@@ -276,37 +276,35 @@ template <class R> __device__ __forceinline__ R radius(R r2) {
   return r2 > R(0) ? sqrt_(r2) : R(0);
 }
 
-// a / b as the product with a reciprocal that is formed once per denominator:
-// quot(a, recip(b)).  In float this is what the approximate division gives, bit for
-// bit, for |b| < 2^126, without the range scaling that each division carries
-// (adjoint pair sweep at 262,144 particles .966 -> .925 ms, 7.46 -> 7.13 ms at
-// 2.1 million); it is for denominators that cannot be larger (squared distances
-// in units of h, radii, parameters).  In double a division is some twenty FP64
-// operations on a pipe that runs at 1/64 of the FP32 rate (adjoint pair sweep of
-// 13,824 particles 4.60 -> 3.64 ms, rates 1.53 -> 1.41 ms).  The product is rounded
-// on its own, never fused.
-__device__ __forceinline__ float recip(float b) {
+// a / b for a denominator that several quotients of a pair share: quot(a, denom(b)).
+// In float denom is the reciprocal, formed once, and the quotient a product, rounded on
+// its own (adjoint pair sweep at 262,144 particles .966 -> .925 ms, 7.46 -> 7.13 ms at
+// 2.1 million); it is for |b| < 2^126 (squared distances in units of h, radii,
+// parameters).  In double denom is b itself and every quotient a division, rounded once:
+// a product with a reciprocal is faster (adjoint pair sweep of 13,824 particles 3.64 ms
+// against 4.60), but errs by .59 units of 2^-53 rms where the division errs by .42, and a
+// power of a reciprocal overflows where the quotient is an ordinary number (the
+// limiter's 4ab / (a + b)^2 below |a + b| = 7.5e-155).
+__device__ __forceinline__ float denom(float b) {
   float y;
   asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(b));
   return y;
 }
-__device__ __forceinline__ double recip(double b) { return 1.0 / b; }
+__device__ __forceinline__ double denom(double b) { return b; }
 __device__ __forceinline__ float quot(float a, float inv) { return __fmul_rn(a, inv); }
-__device__ __forceinline__ double quot(double a, double inv) { return __dmul_rn(a, inv); }
-// a / b for a power b of a denominator, of which p is the same power of the
-// reciprocal.  Double multiplies by p; float takes the reciprocal of b itself, which
-// has the division's bits.
-__device__ __forceinline__ float quot_pow(float a, float b, float) { return quot(a, recip(b)); }
-__device__ __forceinline__ double quot_pow(double a, double, double p) { return quot(a, p); }
-// The same for b = s^2 or s^3 of an s of any size: above 2^41 float scales both sides
+__device__ __forceinline__ double quot(double a, double b) { return a / b; }
+// c + a / b
+__device__ __forceinline__ float add_quot(float c, float a, float inv) {
+  return __fmaf_rn(a, inv, c);
+}
+__device__ __forceinline__ double add_quot(double c, double a, double b) { return c + a / b; }
+// a / b for b = s^2 or s^3 of an s of any size: above 2^41 float scales both sides
 // by 1/4 (exact), so that the reciprocal of a b up to FLT_MAX stays a normal number.
-__device__ __forceinline__ float quot_pow(float a, float b, float, float s) {
+__device__ __forceinline__ float quot_pow(float a, float b, float s) {
   const float k = fabsf(s) > 0x1p41f ? 0.25f : 1.f;
-  return quot(__fmul_rn(a, k), recip(__fmul_rn(b, k)));
+  return quot(__fmul_rn(a, k), denom(__fmul_rn(b, k)));
 }
-__device__ __forceinline__ double quot_pow(double a, double, double p, double) {
-  return quot(a, p);
-}
+__device__ __forceinline__ double quot_pow(double a, double b, double) { return a / b; }
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
 __device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 

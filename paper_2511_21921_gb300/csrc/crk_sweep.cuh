@@ -591,11 +591,11 @@ __device__ __forceinline__ R energy_share(bool split, R E, R ui, R uj) {
 template <class R> struct PairC2 {
   using RC = Rec<R>;
   // limiter phi from a = x.gv_i.x, b = x.gv_j.x:  4ab/(a+b)^2 when ab > 0
-  __device__ static __forceinline__ R limiter_phi(R a, R b, R is) {  // is: recip(a + b)
+  __device__ static __forceinline__ R limiter_phi(R a, R b) {
     const R ab = a * b;
     if (!(ab > R(0))) return R(0);
     const R sm = a + b;
-    return quot_pow(R(4) * ab, sm * sm, is * is, sm);
+    return quot_pow(R(4) * ab, sm * sm, sm);
   }
   template <bool VAR = false>
   __device__ static __forceinline__ void force(const R* ri, const R* rj, const R* d, R r2,
@@ -623,10 +623,10 @@ template <class R> struct PairC2 {
     if (av.limiter) {
       const R pa = d[0] * gix[0] + d[1] * gix[1] + d[2] * gix[2];
       const R pb = d[0] * gjx[0] + d[1] * gjx[1] + d[2] * gjx[2];
-      phi = limiter_phi(pa, pb, recip(pa + pb));
+      phi = limiter_phi(pa, pb);
       const R eta = r * fmin(ihi, ihj);
       if (eta < av.eta_crit) {
-        const R z = quot(eta - av.eta_crit, recip(av.eta_fold));
+        const R z = quot(eta - av.eta_crit, denom(av.eta_fold));
         phi = phi * exp_(-(z * z));
       }
     }
@@ -637,8 +637,8 @@ template <class R> struct PairC2 {
       vh[p] = (ri[RC::C2_VEL + p] - rj[RC::C2_VEL + p]) - hphi * (gix[p] + gjx[p]);
     const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
     const R Di = r2 * (ihi * ihi) + av.eps2, Dj = r2 * (ihj * ihj) + av.eps2;
-    R mui = quot(vx * ihi, recip(Di));
-    R muj = quot(vx * ihj, recip(Dj));
+    R mui = quot(vx * ihi, denom(Di));
+    R muj = quot(vx * ihj, denom(Dj));
     mui = mui < R(0) ? mui : R(0);
     muj = muj < R(0) ? muj : R(0);
     const R Qi = mui * (ri[RC::C2_QB] * mui - ri[RC::C2_QA]);
