@@ -318,10 +318,7 @@ template <class R, bool VAR = false> struct PassA2 {
     R phi = R(0), phi0 = R(0), damp = R(1), z = R(0), pa = R(0), pb = R(0);
     bool dampon = false;
     const R ihmin = fmin(ihi, ihj);
-    // eta and the damping's argument round one by one (rmul, rsub):
-    // the reverse of the limiter is ill conditioned, and every load mode has to give
-    // the same bits whatever the compiler would contract
-    const R eta = rmul(r, ihmin);
+    const R eta = r * ihmin;
     if (a.av.limiter) {
       pa = d[0] * gix[0] + d[1] * gix[1] + d[2] * gix[2];
       pb = d[0] * gjx[0] + d[1] * gjx[1] + d[2] * gjx[2];
@@ -329,7 +326,7 @@ template <class R, bool VAR = false> struct PassA2 {
       phi = phi0;
       if (eta < a.av.eta_crit) {
         dampon = true;
-        z = quot(rsub(eta, a.av.eta_crit), denom(a.av.eta_fold));
+        z = (eta - a.av.eta_crit) / a.av.eta_fold;
         damp = exp_(-(z * z));
         phi = phi0 * damp;
       }
@@ -344,8 +341,7 @@ template <class R, bool VAR = false> struct PassA2 {
     const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
     const R Di = r2 * (ihi * ihi) + a.av.eps2;
     const R Dj = r2 * (ihj * ihj) + a.av.eps2;
-    const R iDi = denom(Di), iDj = denom(Dj);
-    const R tmi = quot(vx * ihi, iDi), tmj = quot(vx * ihj, iDj);
+    const R tmi = vx * ihi / Di, tmj = vx * ihj / Dj;
     const R mui = tmi < R(0) ? tmi : R(0);
     const R muj = tmj < R(0) ? tmj : R(0);
     const R qai = ri[RC::C2_QA], qbi = ri[RC::C2_QB], qaj = rj[RC::C2_QA], qbj = rj[RC::C2_QB];
@@ -433,13 +429,13 @@ template <class R, bool VAR = false> struct PassA2 {
     R vxb = R(0), r2b = R(0), ihib = R(0), rb = R(0);
     R db[3] = {R(0), R(0), R(0)};
     if (tmi < R(0)) {
-      vxb = add_quot(vxb, muib * ihi, iDi);
-      ihib += muib * quot(vx, iDi) * add_quot(R(1), R(-2) * r2 * (ihi * ihi), iDi);
-      r2b += muib * quot(-vx * (ihi * ihi * ihi), denom(Di * Di));
+      vxb += muib * ihi / Di;
+      ihib += muib * (vx / Di) * (R(1) - R(2) * r2 * (ihi * ihi) / Di);
+      r2b += muib * (-vx * (ihi * ihi * ihi) / (Di * Di));
     }
     if (tmj < R(0)) {
-      vxb = add_quot(vxb, mujb * ihj, iDj);
-      r2b += mujb * quot(-vx * (ihj * ihj * ihj), denom(Dj * Dj));
+      vxb += mujb * ihj / Dj;
+      r2b += mujb * (-vx * (ihj * ihj * ihj) / (Dj * Dj));
     }
     R vhb[3], gsum[3];
 #pragma unroll
@@ -459,7 +455,7 @@ template <class R, bool VAR = false> struct PassA2 {
         phi0b = phib * damp;
         const R dampb = phib * phi0;
         const R zb = dampb * (R(-2) * z * damp);
-        const R etab = quot(zb, denom(a.av.eta_fold));
+        const R etab = zb / a.av.eta_fold;
         rb += etab * ihmin;
         const bool own = (ihi < ihj) || (ihi == ihj && st.s < (int64_t)j);
         if (own) ihib += etab * r;
@@ -467,8 +463,8 @@ template <class R, bool VAR = false> struct PassA2 {
       if (pa * pb > R(0)) {
         const R sm = pa + pb;
         const R s3 = sm * sm * sm;
-        const R pab = quot_pow(phi0b * R(4) * pb * (pb - pa), s3, sm);
-        const R pbb = quot_pow(phi0b * R(4) * pa * (pa - pb), s3, sm);
+        const R pab = phi0b * R(4) * pb * (pb - pa) / s3;
+        const R pbb = phi0b * R(4) * pa * (pa - pb) / s3;
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
           db[p] += pab * gix[p] + pbb * gjx[p];
@@ -495,7 +491,7 @@ template <class R, bool VAR = false> struct PassA2 {
     for (int p = 0; p < 3; ++p) db[p] -= ndb[p];
     st.hb += wendland_rev(Wib, gib, Wi, gi, wendland_gg(r, ihi), r2, ihi, d, db);
     (void)wendland_rev(Wjb, gjb, Wj, gj, wendland_gg(r, ihj), r2, ihj, d, db);
-    const R rr = (r > R(0)) ? quot(rb, denom(r)) : R(0);
+    const R rr = (r > R(0)) ? rb / r : R(0);
 #pragma unroll
     for (int p = 0; p < 3; ++p) {
       db[p] += (rr + R(2) * r2b) * d[p];

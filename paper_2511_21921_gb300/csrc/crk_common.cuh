@@ -276,37 +276,7 @@ template <class R> __device__ __forceinline__ R radius(R r2) {
   return r2 > R(0) ? sqrt_(r2) : R(0);
 }
 
-// a / b for a denominator that several quotients of a pair share: quot(a, denom(b)).
-// In float denom is the reciprocal, formed once, and the quotient a product, rounded on
-// its own (adjoint pair sweep at 262,144 particles .966 -> .925 ms, 7.46 -> 7.13 ms at
-// 2.1 million); it is for |b| < 2^126 (squared distances in units of h, radii,
-// parameters).  In double denom is b itself and every quotient a division, rounded once:
-// a product with a reciprocal is faster (adjoint pair sweep of 13,824 particles 3.64 ms
-// against 4.60), but errs by .59 units of 2^-53 rms where the division errs by .42, and a
-// power of a reciprocal overflows where the quotient is an ordinary number (the
-// limiter's 4ab / (a + b)^2 below |a + b| = 7.5e-155).
-__device__ __forceinline__ float denom(float b) {
-  float y;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(b));
-  return y;
-}
-__device__ __forceinline__ double denom(double b) { return b; }
-__device__ __forceinline__ float quot(float a, float inv) { return __fmul_rn(a, inv); }
-__device__ __forceinline__ double quot(double a, double b) { return a / b; }
-// c + a / b
-__device__ __forceinline__ float add_quot(float c, float a, float inv) {
-  return __fmaf_rn(a, inv, c);
-}
-__device__ __forceinline__ double add_quot(double c, double a, double b) { return c + a / b; }
-// a / b for b = s^2 or s^3 of an s of any size: above 2^41 float scales both sides
-// by 1/4 (exact), so that the reciprocal of a b up to FLT_MAX stays a normal number.
-__device__ __forceinline__ float quot_pow(float a, float b, float s) {
-  const float k = fabsf(s) > 0x1p41f ? 0.25f : 1.f;
-  return quot(__fmul_rn(a, k), denom(__fmul_rn(b, k)));
-}
-__device__ __forceinline__ double quot_pow(double a, double b, double) { return a / b; }
 __device__ __forceinline__ float fma_(float a, float b, float c) { return __fmaf_rn(a, b, c); }
-__device__ __forceinline__ double fma_(double a, double b, double c) { return __fma_rn(a, b, c); }
 
 // ---------------------------------------------------------------------------
 // Wendland C4 in 3-D with compact support h (q = r/h):

@@ -82,7 +82,7 @@ inline bool lpt_worthwhile(int64_t items, int64_t warps) {
 //   moments   0.063/0.079/0.327/2.17 -> ring 0.051/0.068, warp ring 0.200/1.32
 //   density   0.059/0.079/0.321/2.11 -> deep buffers 0.047/0.061/0.211/1.40
 //   rates     0.121/0.193/0.600/4.17 -> warp ring 0.100/0.156/0.516/3.74
-//   adjoint   rates 0.165/0.284/1.18/8.64 -> double buffer 0.152/0.254/0.925/7.13
+//   adjoint   rates 0.185/0.310/1.27/9.30 -> double buffer 0.160/0.266/0.966/7.46
 //             density 0.105/0.222/0.641/4.53 -> 0.074/0.174/0.581/4.26
 //             moments 0.102/0.172/0.598/4.14 -> 0.070/0.163/0.566/4.14
 //             volume 0.072/0.091/0.208/1.36 -> 0.047/0.065/0.160/1.24

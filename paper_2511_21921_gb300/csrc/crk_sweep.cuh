@@ -595,7 +595,7 @@ template <class R> struct PairC2 {
     const R ab = a * b;
     if (!(ab > R(0))) return R(0);
     const R sm = a + b;
-    return quot_pow(R(4) * ab, sm * sm, sm);
+    return R(4) * ab / (sm * sm);
   }
   template <bool VAR = false>
   __device__ static __forceinline__ void force(const R* ri, const R* rj, const R* d, R r2,
@@ -626,7 +626,7 @@ template <class R> struct PairC2 {
       phi = limiter_phi(pa, pb);
       const R eta = r * fmin(ihi, ihj);
       if (eta < av.eta_crit) {
-        const R z = quot(eta - av.eta_crit, denom(av.eta_fold));
+        const R z = (eta - av.eta_crit) / av.eta_fold;
         phi = phi * exp_(-(z * z));
       }
     }
@@ -636,9 +636,8 @@ template <class R> struct PairC2 {
     for (int p = 0; p < 3; ++p)
       vh[p] = (ri[RC::C2_VEL + p] - rj[RC::C2_VEL + p]) - hphi * (gix[p] + gjx[p]);
     const R vx = vh[0] * d[0] + vh[1] * d[1] + vh[2] * d[2];
-    const R Di = r2 * (ihi * ihi) + av.eps2, Dj = r2 * (ihj * ihj) + av.eps2;
-    R mui = quot(vx * ihi, denom(Di));
-    R muj = quot(vx * ihj, denom(Dj));
+    R mui = vx * ihi / (r2 * (ihi * ihi) + av.eps2);
+    R muj = vx * ihj / (r2 * (ihj * ihj) + av.eps2);
     mui = mui < R(0) ? mui : R(0);
     muj = muj < R(0) ? muj : R(0);
     const R Qi = mui * (ri[RC::C2_QB] * mui - ri[RC::C2_QA]);
