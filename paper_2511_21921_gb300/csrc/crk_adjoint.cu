@@ -223,6 +223,17 @@ __global__ void k_adj_prep(const R* __restrict__ gdv, const R* __restrict__ gdu,
 // and thread i takes the derivative with respect to its own variables (the
 // share's u_i dependence included; the sign of E_ij is held, as every branch).
 // ===========================================================================
+// Powers of two, so that a change of unit rounds nothing.  The product of pa and pb is a
+// positive number, hence their sum above 2^-63 (float) or 2^-538 (double): in units of
+// 1 / unit its cube and the products beside it are normal numbers.
+template <class R> struct LimiterRange;
+template <> struct LimiterRange<float> {
+  static constexpr double sum = 0x1p-32, unit = 0x1p48;
+};
+template <> struct LimiterRange<double> {
+  static constexpr double sum = 0x1p-300, unit = 0x1p400;
+};
+
 template <class R, bool VAR = false> struct PassA2 {
   // VAR: the formulation variants (per-side viscosity, energy split) are
   // compiled in; the default form is compiled without them so that its
@@ -461,10 +472,18 @@ template <class R, bool VAR = false> struct PassA2 {
         if (own) ihib += etab * r;
       }
       if (pa * pb > R(0)) {
-        const R sm = pa + pb;
+        // the derivatives of phi0 are homogeneous of degree -1 in (pa, pb): below `sum`,
+        // whose cube is near the end of the range, both are taken in units of 1 / `unit`
+        R qa = pa, qb = pb, f = phi0b * R(4);
+        if (fabs(qa + qb) < R(LimiterRange<R>::sum)) {
+          qa *= R(LimiterRange<R>::unit);
+          qb *= R(LimiterRange<R>::unit);
+          f *= R(LimiterRange<R>::unit);
+        }
+        const R sm = qa + qb;
         const R s3 = sm * sm * sm;
-        const R pab = phi0b * R(4) * pb * (pb - pa) / s3;
-        const R pbb = phi0b * R(4) * pa * (pa - pb) / s3;
+        const R pab = f * qb * (qb - qa) / s3;
+        const R pbb = f * qa * (qa - qb) / s3;
 #pragma unroll
         for (int p = 0; p < 3; ++p) {
           db[p] += pab * gix[p] + pbb * gjx[p];
