@@ -628,14 +628,15 @@ __device__ __forceinline__ double sq(double a) { return __dmul_rn(a, a); }
 // at most 3 * 2^-24 h^2 (one rounding, and in the FP64 form h rounded to
 // float).  A decision r^2 < h^2 is therefore certain outside the band
 // |r^2 - h^2| <= tol(h) below (wider by a third in the L term and more in the
-// h^2 term); inside it the pair is decided again in double exactly as the
-// definition states -- minimum image decided and formed in double, r^2 summed
-// without contraction, compared with the squared smoothing lengths -- so the
-// lists of both forms are those of the double predicate.  (Testing every
-// candidate of the FP64 form in double took 2.89 ms of its build on 13,824
-// particles: GB300 runs FP64 at 1/64 of the FP32 rate.)
+// h^2 term, and by 2^-123 for what the five operations on the way flush to 0, each
+// less than 2^-126: it is never 0, so equality of two flushed values is uncertain);
+// inside it the pair is decided again in double exactly as the definition states --
+// minimum image decided and formed in double, r^2 summed without contraction, compared
+// with the squared smoothing lengths -- so the lists of both forms are those of the
+// double predicate.  (Testing every candidate of the FP64 form in double took 2.89 ms
+// of its build on 13,824 particles: GB300 runs FP64 at 1/64 of the FP32 rate.)
 __device__ __forceinline__ float list_band(float h, float L) {
-  return 5.9604645e-8f * fmaf(16.f * h, h, 24.f * L * h);
+  return 0x1p-24f * fmaf(16.f * h, h, fmaf(24.f * L, h, 0x1p-99f));
 }
 __device__ __forceinline__ double exact_r2(const double* __restrict__ xd, int64_t n, int64_t pi,
                                            int64_t pj, double L) {
