@@ -381,7 +381,9 @@ crk_status crk_cool_exact(crk_plan* plan, crk_stream_t stream, int64_t n,
  * every sweep with CUDA events and keeps the fastest variant per sweep in the
  * plan.  Outputs of the trial runs go to the workspace; afterwards the
  * workspace holds the state of a complete crk_moments + crk_rates call.
- * choice_out (optional, host int32[8]) receives the chosen variant per sweep,
+ * A sweep that was not timed (the adjoint's without cotangents, all of them for n = 0 or
+ * after an error) keeps the choice it had, or none.
+ * choice_out (optional, host int32[8]) receives the variant each sweep now takes,
  * ms_out (optional, host float[8][CRK_TUNE_VARIANTS]) the mean milliseconds of
  * every variant.  Synchronises.  Requires a built workspace.  A plan that was
  * neither tuned nor given choices takes a variant by sweep, precision and size. */

@@ -519,6 +519,8 @@ crk_status crk_autotune(crk_plan* plan, crk_stream_t stream, void* ws, const voi
   static const int queues[8] = {Q_B1, Q_B2, Q_C1, Q_C2, Q_A_C2, Q_A_C1, Q_A_B2, Q_A_B1};
   double tsum[8][CRK_TUNE_VARIANTS] = {};
   const bool was_timing = P.timing;
+  int before[8];
+  for (int q = 0; q < 8; ++q) before[q] = P.variant[queues[q]];
   auto run = [&]() -> crk_status {
     crk_status r;
     if (P.p.precision == CRK_FP64) {
@@ -571,11 +573,11 @@ crk_status crk_autotune(crk_plan* plan, crk_stream_t stream, void* ws, const voi
     int best = 0;
     for (int k = 1; k < CRK_TUNE_VARIANTS; ++k)
       if (tsum[q][k] > 0 && tsum[q][k] < tsum[q][best]) best = k;
-    // a sweep that was not timed keeps the rule's variant
-    if (s != CRK_OK || (q >= 4 && !adj))
-      best = default_variant(queues[q], P.p.precision, P.ly.n);
-    P.variant[queues[q]] = best;
-    if (choice_out) choice_out[q] = best;
+    // a sweep that was not timed keeps what the plan had: a choice, or the rule, which
+    // follows the size of later builds
+    const bool timed = s == CRK_OK && tsum[q][best] > 0;
+    P.variant[queues[q]] = timed ? best : before[q];
+    if (choice_out) choice_out[q] = variant_of(P, queues[q]);
     if (ms_out)
       for (int k = 0; k < CRK_TUNE_VARIANTS; ++k)
         ms_out[q * CRK_TUNE_VARIANTS + k] = (float)(tsum[q][k] / repeats);

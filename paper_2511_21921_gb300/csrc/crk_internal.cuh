@@ -104,6 +104,12 @@ inline int default_variant(int queue, int precision, int64_t n) {
   }
 }
 
+// The variant a sweep of this plan takes now: the one chosen, or the rule's.
+inline int variant_of(const Plan& plan, int queue) {
+  const int v = plan.variant[queue];
+  return v != Plan::kAutoVariant ? v : default_variant(queue, plan.p.precision, plan.ly.n);
+}
+
 template <class R>
 crk_status cell_build_impl(Plan* plan, cudaStream_t st, char* ws, int64_t n, int32_t nb,
                            const int64_t* box_off, const double* box_L, const double* x,

@@ -695,10 +695,7 @@ void launch_sweep_plain(Plan* plan, cudaStream_t st, const typename P::Args& a, 
 // lane groups).
 template <class P>
 void launch_sweep(Plan* plan, cudaStream_t st, const typename P::Args& a, const char* name) {
-  const int chosen = plan->variant[P::QUEUE];
-  const int v = chosen != Plan::kAutoVariant
-                    ? chosen
-                    : default_variant(P::QUEUE, plan->p.precision, plan->ly.n);
+  const int v = variant_of(*plan, P::QUEUE);
   Phase ph(plan, st, name, 1);
   switch (v) {
     case 1: launch_variant<P, P::MB1, 0>(plan, st, a); break;
