@@ -329,7 +329,11 @@ template <class R, bool VAR = false> struct PassA2 {
     R phi = R(0), phi0 = R(0), damp = R(1), z = R(0), pa = R(0), pb = R(0);
     bool dampon = false;
     const R ihmin = fmin(ihi, ihj);
-    const R eta = r * ihmin;
+    // eta and the damping's argument round one by one in float: the reverse of the
+    // limiter is ill conditioned, and the load modes have to give the same bits whatever
+    // the compiler would contract in each
+    constexpr bool PIN = sizeof(R) == 4;
+    const R eta = PIN ? rmul(r, ihmin) : r * ihmin;
     if (a.av.limiter) {
       pa = d[0] * gix[0] + d[1] * gix[1] + d[2] * gix[2];
       pb = d[0] * gjx[0] + d[1] * gjx[1] + d[2] * gjx[2];
@@ -337,7 +341,7 @@ template <class R, bool VAR = false> struct PassA2 {
       phi = phi0;
       if (eta < a.av.eta_crit) {
         dampon = true;
-        z = (eta - a.av.eta_crit) / a.av.eta_fold;
+        z = (PIN ? rsub(eta, a.av.eta_crit) : eta - a.av.eta_crit) / a.av.eta_fold;
         damp = exp_(-(z * z));
         phi = phi0 * damp;
       }
