@@ -96,8 +96,9 @@ typedef struct {
   int32_t nbr_cap;  /* neighbor-list slots per particle reserved in the workspace; 0 = 192 */
   int32_t block_threads; /* threads per block of the pair sweeps; 0 = autotuned default */
   int32_t blocks_per_sm; /* resident blocks per SM for the persistent sweeps; 0 = default */
-  int32_t prefetch;      /* sweeps prefetch the neighbor record this many list entries ahead
-                            into L1; 0 = off */
+  int32_t prefetch;      /* 1..16: sweeps with plain loads (launch variants 0-2) prefetch the
+                            neighbor record this many list entries ahead into L1; 0 = off.
+                            The other variants fetch ahead by themselves and ignore it */
   int32_t energy_split;  /* compatible energy split of the pair work E_ij = m_i a_ij.(v_j - v_i)
                             (Sec. 2.1): 0 = halves, f_ij = 1/2; 1 = weighted by the specific
                             energies, f_ij = (1 + sgn(E_ij)(u_j - u_i)/(u_i + u_j))/2, so heating

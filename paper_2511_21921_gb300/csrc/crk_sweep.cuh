@@ -18,7 +18,7 @@ struct Common {
   const double* __restrict__ box_L;
   const int32_t* __restrict__ perm;
   int64_t cap_pp;  // list slots per particle: gather part, then the scatter-only entries
-  int pf;          // prefetch distance in list entries (0 = off)
+  int pf;          // prefetch distance of the plain loads in list entries (0 = off)
   // optional compacted work list of the active-set sweeps (sorted indices; its
   // length on the device): warps then take 32 listed particles per item
   // instead of 32 consecutive ones
@@ -395,13 +395,14 @@ __global__ void __launch_bounds__(P::BLOCK) __maxnreg__(sweep_regs(P::BLOCK, MIN
       auto raw = [&](int k) -> uint32_t { return k < tot ? __ldg(col + (int64_t)k * 32) : 0u; };
 #pragma unroll
       for (int i = 0; i < kAhead; ++i) e[i] = raw(i);
-      const bool pf = a.c.pf > 0;
+      const int pf = a.c.pf;
       for (int k = 0; k < wmax; ++k) {
         const uint32_t ek = e[0];
 #pragma unroll
         for (int i = 0; i + 1 < kAhead; ++i) e[i] = e[i + 1];
         e[kAhead - 1] = raw(k + kAhead);
-        if (pf && k + 1 < tot) prefetch_sources<P>(a, e[0] & kIdxMask);
+        if (pf && k + pf < tot)
+          prefetch_sources<P>(a, __ldg(col + (int64_t)(k + pf) * 32) & kIdxMask);
         if (k < tot && index_ok(a.c.hdr, ek & kIdxMask, a.c.n)) {
           Real r0[P::SW0], r1[P::SW1 > 0 ? P::SW1 : 1];
           load_sources<P>(a, ek & kIdxMask, r0, r1);
