@@ -673,9 +673,15 @@ void launch_variant(Plan* plan, cudaStream_t st, const typename P::Args& a) {
   // a box of few items is spread over all multiprocessors in smaller blocks (the
   // ring keeps its stride): 13,824 particles are 432 items, 54 blocks of 256;
   // their FP64 volume, moment and density sweeps went 0.32, 0.79, 0.81 ->
-  // 0.20, 0.45, 0.45 ms, the mixed moments of 4096 particles 0.039 -> 0.033
+  // 0.20, 0.45, 0.45 ms, the mixed moments of 4096 particles 0.039 -> 0.033.
+  // Where blocks_per_sm limits the blocks, only while the smaller ones still hold all
+  // items at once (one block a SM, 8,000 particles: moments 0.086 ms, and 0.139 with 152
+  // blocks of one warp for 250 items)
   int block = P::BLOCK;
-  while (block > 32 && plan->ly.nw * 32 < (int64_t)block * plan->num_sms) block /= 2;
+  const int64_t threads = plan->ly.nw * 32, sms = plan->num_sms, limit = plan->p.blocks_per_sm;
+  while (block > 32 && threads < block * sms &&
+         (limit == 0 || threads <= block / 2 * sms * limit))
+    block /= 2;
   const int grid = sweep_grid(plan, fn, block, (int)smem);
   typename P::Args b = a;
   b.c.lpt = P::LPT && lpt_worthwhile(plan->ly.nw, (int64_t)grid * block / 32);
