@@ -30,7 +30,7 @@ Layout make_layout(const crk_params& p, int64_t n, int32_t nb) {
   const int B2 = p.precision == CRK_FP64 ? Rec<double>::B2 : Rec<float>::B2;
   const int C1 = p.precision == CRK_FP64 ? Rec<double>::C1 : Rec<float>::C1;
   const int C2 = p.precision == CRK_FP64 ? Rec<double>::C2 : Rec<float>::C2;
-  const size_t N = (size_t)n, NT = (size_t)L.nt, NI = (size_t)std::max<int64_t>(L.ni, 1);
+  const size_t N = (size_t)n, NT = (size_t)L.nt;
   const size_t NW = (size_t)L.nw;
   size_t o = 0;
   auto take = [&o](size_t bytes) {

@@ -704,11 +704,11 @@ constexpr int kStage = 96;
 template <class R>
 __global__ void __launch_bounds__(32, kNbrBlocks) k_nbr(
     const uint64_t* __restrict__ keys, const R* __restrict__ hs, const int32_t* __restrict__ boxid,
-    const double* __restrict__ box_L, int64_t n, int64_t nbk, int64_t ni, int64_t nt,
-    const float* __restrict__ nrec, const float4* __restrict__ p4, int32_t* __restrict__ cnt_g, int32_t* __restrict__ cnt_s, int32_t* __restrict__ wlen_g,
-    int32_t* __restrict__ wlen_s, uint32_t* __restrict__ ell, int64_t cap_pp, DevHeader* hdr,
-    const double* __restrict__ xd, const int32_t* __restrict__ perm,
-    const float* __restrict__ hbox) {
+    const double* __restrict__ box_L, int64_t n, int64_t ni, const float* __restrict__ nrec,
+    const float4* __restrict__ p4, int32_t* __restrict__ cnt_g, int32_t* __restrict__ cnt_s,
+    int32_t* __restrict__ wlen_g, int32_t* __restrict__ wlen_s, uint32_t* __restrict__ ell,
+    int64_t cap_pp, DevHeader* hdr, const double* __restrict__ xd,
+    const int32_t* __restrict__ perm, const float* __restrict__ hbox) {
   __shared__ int32_t stk[kNodeStack];
   // candidate buckets; the top bit marks one that may hold particles of two boxes
   __shared__ int32_t cand[64];
@@ -1299,7 +1299,7 @@ crk_status cell_build_impl(Plan* plan, cudaStream_t st, char* ws, int64_t n, int
   R* xs = reinterpret_cast<R*>(ws + Ly.xs);
   R* hs = reinterpret_cast<R*>(ws + Ly.hs);
   ph_sort.end();
-  const int64_t nbk = Ly.nbk, ni = Ly.ni, nt = Ly.nt;
+  const int64_t nbk = Ly.nbk, ni = Ly.ni;
   // the segment tree lives in the region of the rate records, which hold nothing
   // between a build's start and the sweeps that write them
   SegTree seg{};
@@ -1331,9 +1331,9 @@ crk_status cell_build_impl(Plan* plan, cudaStream_t st, char* ws, int64_t n, int
   int32_t* wlen_g = reinterpret_cast<int32_t*>(ws + Ly.wlen_g);
   int32_t* wlen_s = reinterpret_cast<int32_t*>(ws + Ly.wlen_s);
   uint32_t* ell = reinterpret_cast<uint32_t*>(ws + Ly.ell);
-  k_nbr<R><<<(unsigned)Ly.nw, 32, 0, st>>>(k0, hs, boxid, wbox, n, nbk, ni, nt, nrec, p4, cnt_g,
-                                             cnt_s, wlen_g, wlen_s, ell, Ly.cap_pp, hdr, x, perm,
-                                             reinterpret_cast<const float*>(hbox));
+  k_nbr<R><<<(unsigned)Ly.nw, 32, 0, st>>>(k0, hs, boxid, wbox, n, ni, nrec, p4, cnt_g, cnt_s,
+                                           wlen_g, wlen_s, ell, Ly.cap_pp, hdr, x, perm,
+                                           reinterpret_cast<const float*>(hbox));
   int32_t* cost = reinterpret_cast<int32_t*>(ws + Ly.item_cost);
   int32_t* seq_cost = reinterpret_cast<int32_t*>(ws + Ly.seq_cost);
   k_balance<<<(unsigned)((n + kBalance - 1) / kBalance), kBalance, 0, st>>>(

@@ -17,11 +17,9 @@ constexpr int kBucket = 8;          // particles per tree leaf (bucket)
 constexpr int kSortTile = 1024;     // keys per radix-sort tile (small: enough blocks to fill the GPU)
 constexpr int kSortThreads = 256;
 constexpr int kNodeRec = 16;        // words per packed tree-node record (64 bytes)
-constexpr int kStackDepth = 96;     // tree traversal stack (depth <= 64 key bits + 30 index bits)
 constexpr uint32_t kIdxMask = 0x3fffffffu;
 constexpr uint32_t kGatherBit = 0x80000000u;   // j in G(i):  r < h_i
 constexpr uint32_t kScatterBit = 0x40000000u;  // i in G(j):  r < h_j
-constexpr uint32_t kSentinel = 0xffffffffu;
 
 // Work-queue counters, one per persistent sweep of a call.
 enum Queue {

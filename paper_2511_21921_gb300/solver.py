@@ -425,7 +425,10 @@ class Solver:
 
 class CRKRates(torch.autograd.Function):
     """(dv/dt, du/dt) = CRKSPH rates of (x, v, u, h) with masses m; the backward
-    pass is libcrk's adjoint (no per-pair storage; forward state is reused)."""
+    pass is libcrk's adjoint over the lists of the forward pass (no per-pair storage;
+    volumes, moments and densities are evaluated again, since other calls of the same
+    solver may have replaced them).  The lists have to be those of the forward pass: no
+    other build of this solver may come between."""
 
     @staticmethod
     def forward(ctx, x, v, u, h, m, solver: Solver, box_off=None, box_L=None, L_box=1.0):
