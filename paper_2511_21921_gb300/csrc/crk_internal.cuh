@@ -95,9 +95,9 @@ inline bool lpt_worthwhile(int64_t items, int64_t warps) {
 // contract different products in each, so that variants agree to rounding in general;
 // those taken here gave the bits of plain loads at every size measured (4 k to 2.1 M).
 // The figures are of full sweeps; active-set sweeps choose by the box's n as well
-// (shares of .3 % to 100 % of 4 k, 30 k and 262 k particles all ran 1.5-2.2 times
-// as fast as plain loads did before).  The FP64 form is bound by its pipe: every
-// variant is within 5 % of plain loads.
+// (shares of .3 % to 100 % of 4 k, 30 k and 262 k particles: 1.4-2.2 times as fast as
+// with the plain loads before it).  The FP64 form is bound by its pipe: the best variant
+// of a sweep is within 10 % of plain loads (adjoint volume 14 % at 110 k particles).
 inline int default_variant(int queue, int precision, int64_t n) {
   if (precision == CRK_FP64) return 0;
   switch (queue) {
